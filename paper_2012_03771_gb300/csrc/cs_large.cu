@@ -437,56 +437,20 @@ __device__ __forceinline__ void walk_warp(const LargeArgs &a, TGItem<MT> *q, con
                         dk[k] = dd;
                         vk[k] = big_q ? mul_add_mod(vv, r, dd, pp, fq) : add_times(vv, r, dd, pp);
                     }
-                    // the two steps from one run of Euclid's algorithm on (p, r');
-                    // for 64-bit primes and 2SL >= 1024 mostly in 32-bit steps
-                    if constexpr (sizeof(UT) == 8) {
-                        if (w >= 1024) {
-                            uint64_t a64, b64;
-                            uint32_t da32, ub32;
-                            ok = tg_steps_w(pp, rq, (uint32_t)w, a64, da32, b64, ub32, it, max_iter);
-                            ma_ = a64; mb_ = b64; da_ = da32; ub_ = ub32;
-                        } else {
-                            ok = tg_steps<UT>(pp, rq, w, ma_, da_, mb_, ub_, it, max_iter);
-                        }
-                    } else {
-                        ok = tg_steps<UT>(pp, rq, w, ma_, da_, mb_, ub_, it, max_iter);
-                    }
+                    // the two steps from one run of Euclid's algorithm on (p, r')
+                    ok = walker_steps<UT>(pp, rq, w, ma_, da_, mb_, ub_, it, max_iter);
                     if (!ok) c.err |= ERR_SOLVER_LIMIT;
                     uint32_t n_first = 0;
 #pragma unroll
                     for (int k = 0; k < NC; k++) n_first += vk[k] > w;
                     c.solves += 2 + n_first;
-                    if constexpr (sizeof(UT) == 4) {
-                        // each walker's first hit from the step basis, without a solve
+                    // each walker's first hit from the step basis, without a solve
+                    if (ok && n_first) {
+                        const float fp = walker_rcp(pp);
 #pragma unroll
-                        for (int k = 0; k < NC; k++) {
-                            if (ok && vk[k] > w) {
-                                uint32_t y;
-                                first[k] = (uint64_t)first_hit32(pp, fq, w, ma_, da_, mb_, ub_, vk[k], y) * Q;
-                                vk[k] = y;
-                            }
-                        }
-                    } else if (ok && n_first) {
-                        // 64-bit (p < 2^40, 2SL <= 2^21): the same with 64-bit
-                        // products (first_hit_w) when both steps are below 2^31 and
-                        // 2SL >= 1024, else with 128-bit ones (first_hit64)
-                        const bool narrow_ab = w >= 1024 && ((uint64_t)ma_ | (uint64_t)mb_) < (1ull << 31);
-                        const float fp = rcp_rn(u64_to_f((uint64_t)pp));
-#pragma unroll
-                        for (int k = 0; k < NC; k++) {
-                            if (vk[k] > w) {
-                                if (narrow_ab) {
-                                    uint32_t y;
-                                    first[k] = first_hit_w(pp, fp, (uint32_t)w, (uint32_t)ma_, (uint32_t)da_,
-                                                           (uint32_t)mb_, (uint32_t)ub_, vk[k], y) * Q;
-                                    vk[k] = (UT)y;
-                                } else {
-                                    uint64_t y;
-                                    first[k] = first_hit64(pp, w, ma_, da_, mb_, ub_, vk[k], y) * Q;
-                                    vk[k] = (UT)y;
-                                }
-                            }
-                        }
+                        for (int k = 0; k < NC; k++)
+                            if (vk[k] > w)
+                                first[k] = walker_first_hit<UT>(pp, fp, w, ma_, da_, mb_, ub_, vk[k]) * Q;
                     }
                 }
                 c.levels += it;
