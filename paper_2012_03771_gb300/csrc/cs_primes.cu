@@ -8,10 +8,16 @@
 // (grid-stride over segments).  The multiples of 3..31 come from tabulated
 // period masks; those of the other base primes q <= sqrt(hi) are marked with
 // shared-memory atomics: small q cooperatively by a warp, large q one per
-// thread.  Each warp then scans its share of the segment, queues the
-// primes it finds in shared memory and, 32 at a time, computes K mod p with
-// Montgomery multiplication over K's prime factors packed into machine words,
-// and appends the entries to the output with one atomic per 32 primes.
+// thread, their first multiples from float quotients.  The CTA takes the output
+// entries of a whole segment with one atomic; each warp then scans its share of
+// the segment, queues the primes it finds in shared memory and, 32 at a time,
+// computes K mod p with Montgomery multiplication over K's prime factors packed
+// into machine words (64-bit primes: the residue kernel after the sieve) and
+// writes the entries.
+//
+// Bound: instruction issue.  Per prime near 9e9, about 16 marks (a shared-memory
+// atomic and five instructions each), the first multiples of the base primes
+// (twenty instructions each, per segment) and the extraction.
 #include <atomic>
 
 #include "cs_arith.cuh"
@@ -21,35 +27,28 @@ namespace cs {
 
 namespace {
 
-// odd numbers per segment (maximum), and the base primes marked by a whole
-// warp (below) or one thread each (above): a warp's lanes on multiples of one
-// q >= 1024 fall on few shared-memory banks, one q per lane spreads them
-// (1024 measured best of 128 to 16384)
-#ifndef CS_GEN_SEG_LOG
-#define CS_GEN_SEG_LOG 17
-#endif
-#ifndef CS_WARP_COOP_Q
-#define CS_WARP_COOP_Q 1024
-#endif
-// grid of the generator: CTAs per SM, and segments per CTA it is sized for
-#ifndef CS_GEN_GRID_PER_SM
-#define CS_GEN_GRID_PER_SM 8
-#endif
-#ifndef CS_GEN_SEGS_PER_CTA
-#define CS_GEN_SEGS_PER_CTA 1
-#endif
-// 1: grid of the resident CTAs and segments sized for whole waves of them
-#ifndef CS_GEN_ONE_WAVE
-#define CS_GEN_ONE_WAVE 1
-#endif
-constexpr uint32_t SEG = 1u << CS_GEN_SEG_LOG;
-constexpr uint32_t SEG_MIN = 1u << 12;      // smallest segment: 8 warps x 16-word batches
+// base primes marked by a whole warp (below) or one thread each (above): a
+// warp's lanes on multiples of one q >= 1024 fall on few shared-memory banks, one
+// q per lane spreads them (1024 measured best of 128 to 16384)
+constexpr uint32_t WARP_COOP_Q = 1024;
+constexpr uint32_t N_COOP = 171;            // odd primes below it: the ascending base list reaches it there
+// Every segment computes the first multiple of every base prime, whose number
+// grows with sqrt(hi) (26,000 at 9e10), so segments are large: up to 2^18 odd
+// numbers, two CTAs of 1024 threads per SM.  A list of the primes of 2^27 numbers
+// at 9e8 / 9e9 / 9e10 takes 51 / 57 / 69 us (54 / 63 / 85 with four CTAs of 512
+// threads, 61 / 76 / 107 with five of 256 and 2^17 odd numbers).
+constexpr int GEN_MIN_BLOCKS = 2;
+constexpr uint32_t SEG = 1u << 18;
+constexpr uint32_t SEG_MIN = 1u << 10;      // smallest segment: 32 words
 constexpr uint32_t SEG_WORDS = SEG / 32;
-constexpr uint32_t GEN_THREADS = 256;
+constexpr uint32_t GEN_THREADS = 1024;
 constexpr uint32_t GEN_WARPS = GEN_THREADS / 32;
-constexpr uint32_t WARP_COOP_Q = CS_WARP_COOP_Q;
-constexpr uint32_t BATCH = 16;              // words scanned per warp step (lanes 0..15)
-constexpr uint32_t QCAP = BATCH * 32 + 32;  // per-warp queue (odd indices within the segment)
+// per-warp queue: the primes of one step (32 words, 2048 consecutive numbers: at
+// most 2 * 2048 / log 2048 = 537 by Montgomery and Vaughan) and 31 left over; kept
+// as 16-bit positions in the warp's part of the segment
+constexpr uint32_t QCAP = 576;
+static_assert(SEG / GEN_WARPS <= 65536, "16-bit positions");
+static_assert(SEG_MIN % (32 * GEN_WARPS) == 0, "whole words per warp");
 
 // SMALL: tile records; LARGE32/64: (p, r, v0) of one plan; LIST: p only;
 // PR32/64: (p, r) for a residue cache shared by plans with the same K
@@ -107,8 +106,9 @@ __device__ __forceinline__ uint64_t kmodp64(uint64_t p, uint64_t pinv, uint64_t 
     return acc;
 }
 
+// slot: the output entry of this lane's prime
 template <int KIND>
-__device__ __forceinline__ void emit(const GenArgs &a, uint64_t p, bool valid, unsigned lane) {
+__device__ __forceinline__ void emit(const GenArgs &a, uint64_t p, bool valid, uint64_t slot) {
     // residue work for this lane's prime
     uint32_t e0 = 0, e1 = 0, e2 = 0, e3 = 0;
     uint64_t w0 = 0, w1 = 0;
@@ -151,15 +151,7 @@ __device__ __forceinline__ void emit(const GenArgs &a, uint64_t p, bool valid, u
             w0 = p;
         }
     }
-    unsigned mask = __ballot_sync(0xffffffffu, valid);
-    unsigned n = __popc(mask);
-    if (n == 0) return;
-    unsigned long long base = 0;
-    if (lane == 0) base = atomicAdd(a.count, (unsigned long long)n);
-    base = __shfl_sync(0xffffffffu, base, 0);
-    unsigned rank = __popc(mask & ((1u << lane) - 1));
     if (!valid) return;
-    uint64_t slot = base + rank;
     if (slot >= a.cap) {
         atomicOr(a.err, (unsigned long long)ERR_PRIME_OVERFLOW);
         return;
@@ -250,55 +242,75 @@ __device__ __forceinline__ uint32_t first_rem(uint64_t n, uint32_t q) {
     return (n >> 32) == 0 ? (uint32_t)n % q : (uint32_t)(n % q);
 }
 
-// Pre-sieve of the odd multiples of 3..31 (half of all marks, and the ones
-// whose lanes collide on the same shared-memory word): the masks of one period
-// of T = 3*5*7, 11*13, 17*19, 23*29 and 31 odd indices are tabulated in shared
-// memory, and word w of a segment, whose first odd index I = i0 + 32 w has
-// I mod T = s, ORs in table entry s.  Bit b of that entry is set when the odd
-// number 2(I + b) + 1 has a factor q | T, i.e. I + b = (q - 1)/2 (mod q).
-constexpr int PRE_N = 5;
-constexpr uint32_t PRE_MAX_Q = 31;
-__device__ __constant__ uint32_t c_pre_T[PRE_N] = {105, 143, 323, 667, 31};
-__device__ __constant__ uint32_t c_pre_off[PRE_N + 1] = {0, 105, 248, 571, 1238, 1269};
-constexpr uint32_t PRE_WORDS = 1269;
-
-__device__ __forceinline__ uint32_t pre_mask(uint32_t T, uint32_t s) {
-    const uint32_t qs[10] = {3, 5, 7, 11, 13, 17, 19, 23, 29, 31};
-    uint32_t m = 0;
-#pragma unroll
-    for (int k = 0; k < 10; k++) {
-        const uint32_t q = qs[k];
-        if (T % q) continue;
-        const uint32_t h = (q - 1) / 2;
-        for (uint32_t b = (h + q - s % q) % q; b < 32; b += q) m |= 1u << b;
-    }
-    return m;
+// Smallest k >= 0 with q | 2 (i0 + k) + 1, for odd 1024 <= q < 2^21 and i0 < 2^40
+// (fi0 = i0 rounded to float): i0 + k = (q - 1)/2 (mod q).  i0 mod q from two float
+// quotients without a 64-bit division: the first, i0 / q < 2^30, is off by less
+// than 2^7 (three roundings of 2^-23 at most), so i0 less its multiple of q fits
+// 32 signed bits and is taken modulo 2^32; the second, rounded, leaves a
+// remainder within q/2 + 1 of 0.
+__device__ __forceinline__ uint32_t first_multiple(uint64_t i0, float fi0, uint32_t q) {
+    const float rq = rcp_approx((float)q);
+    const uint32_t q1 = (uint32_t)(fi0 * rq);
+    const int32_t r1 = (int32_t)((uint32_t)i0 - q1 * q);
+    const int32_t q2 = __float2int_rn((float)r1 * rq);
+    int32_t r = r1 - q2 * (int32_t)q;
+    if (r < 0) r += (int32_t)q;
+    int32_t k = (int32_t)(q >> 1) - r;
+    if (k < 0) k += (int32_t)q;
+    return (uint32_t)k;
 }
 
+// Pre-sieve of the odd multiples of 3..31 (half of all marks, and the ones
+// whose lanes collide on the same shared-memory word): the masks of one period
+// of T = 3*5*7, 11*13, 17*19, 23*29 and 31 odd indices are tabulated, and word w
+// of a segment, whose first odd index I = i0 + 32 w has I mod T = s, ORs in table
+// entry s.  Bit b of that entry is set when the odd number 2(I + b) + 1 has a
+// factor q | T, i.e. I + b = (q - 1)/2 (mod q).  The tables are computed at
+// compile time and copied to shared memory (computing them in every CTA cost
+// about a seventh of a light chunk's generation).
+constexpr int PRE_N = 5;
+constexpr uint32_t PRE_MAX_Q = 31;
+CS_HD constexpr uint32_t pre_T(int t) { return t == 0 ? 105 : t == 1 ? 143 : t == 2 ? 323 : t == 3 ? 667 : 31; }
+CS_HD constexpr uint32_t pre_off(int t) {
+    return t == 0 ? 0 : t == 1 ? 105 : t == 2 ? 248 : t == 3 ? 571 : t == 4 ? 1238 : 1269;
+}
+constexpr uint32_t PRE_WORDS = 1269;
+struct PreTable {
+    uint32_t w[PRE_WORDS];
+};
+constexpr PreTable make_pre_table() {
+    PreTable t{};
+    constexpr uint32_t qs[10] = {3, 5, 7, 11, 13, 17, 19, 23, 29, 31};
+    for (int k = 0; k < PRE_N; k++)
+        for (uint32_t s = 0; s < pre_T(k); s++) {
+            uint32_t m = 0;
+            for (int j = 0; j < 10; j++) {
+                const uint32_t q = qs[j];
+                if (pre_T(k) % q) continue;
+                for (uint32_t b = ((q - 1) / 2 + q - s % q) % q; b < 32; b += q) m |= 1u << b;
+            }
+            t.w[pre_off(k) + s] = m;
+        }
+    return t;
+}
+__device__ const PreTable c_pre = make_pre_table();
+
 template <int KIND>
-__global__ void __launch_bounds__(GEN_THREADS) k_gen(const GenArgs a) {
-    __shared__ uint32_t comp[SEG_WORDS];          // bit set = composite (or out of range)
-    __shared__ uint32_t queue[GEN_WARPS][QCAP];
-    __shared__ uint32_t pre[PRE_WORDS];           // pre-sieve tables
+__global__ void __launch_bounds__(GEN_THREADS, GEN_MIN_BLOCKS) k_gen(const GenArgs a) {
+    extern __shared__ uint32_t gen_smem[];
+    uint32_t *comp = gen_smem;                    // SEG_WORDS: bit set = composite (or out of range)
+    uint32_t *pre = comp + SEG_WORDS;             // PRE_WORDS: pre-sieve tables
+    uint16_t *queue = reinterpret_cast<uint16_t *>(pre + PRE_WORDS) + (threadIdx.x >> 5) * QCAP;
+    __shared__ uint32_t warp_n[GEN_WARPS];        // primes in each warp's part of the segment
+    __shared__ unsigned long long seg_base;       // output entry of the segment's first prime
     const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (uint32_t e = threadIdx.x; e < PRE_WORDS; e += GEN_THREADS) {
-        int t = 0;
-        while (e >= c_pre_off[t + 1]) t++;
-        pre[e] = pre_mask(c_pre_T[t], e - c_pre_off[t]);
-    }
+    for (uint32_t e = threadIdx.x; e < PRE_WORDS; e += GEN_THREADS) pre[e] = c_pre.w[e];
     __syncthreads();
 
-    if (a.emit_two && blockIdx.x == 0 && warp == 0) emit<KIND>(a, 2, lane == 0, lane);
+    if (a.emit_two && blockIdx.x == 0 && threadIdx.x == 0)
+        emit<KIND>(a, 2, true, atomicAdd(a.count, 1ull));
 
-    // first base index with q >= WARP_COOP_Q (base is ascending)
-    uint32_t big0 = 0;
-    {
-        uint32_t hi = a.n_base;
-        while (big0 < hi) {
-            uint32_t mid = (big0 + hi) / 2;
-            if (__ldg(&a.base[mid]) < WARP_COOP_Q) big0 = mid + 1; else hi = mid;
-        }
-    }
+    const uint32_t n_coop = min(N_COOP, a.n_base);   // base primes marked by whole warps
 
     for (uint64_t s = blockIdx.x; s < a.n_seg; s += gridDim.x) {
         const uint64_t i0 = a.i_begin + s * a.seg;
@@ -312,7 +324,7 @@ __global__ void __launch_bounds__(GEN_THREADS) k_gen(const GenArgs a) {
         uint32_t ph[PRE_N], step[PRE_N];
 #pragma unroll
         for (int t = 0; t < PRE_N; t++) {
-            const uint32_t T = c_pre_T[t];
+            const uint32_t T = pre_T(t);
             ph[t] = pre_ok ? first_rem(i0 + 32ull * threadIdx.x, T) : 0;
             step[t] = (32u * GEN_THREADS) % T;
         }
@@ -323,9 +335,9 @@ __global__ void __launch_bounds__(GEN_THREADS) k_gen(const GenArgs a) {
             if (pre_ok) {
 #pragma unroll
                 for (int t = 0; t < PRE_N; t++) {
-                    v |= pre[c_pre_off[t] + ph[t]];
+                    v |= pre[pre_off(t) + ph[t]];
                     ph[t] += step[t];
-                    if (ph[t] >= c_pre_T[t]) ph[t] -= c_pre_T[t];
+                    if (ph[t] >= pre_T(t)) ph[t] -= pre_T(t);
                 }
             }
             comp[w] = v;
@@ -333,95 +345,122 @@ __global__ void __launch_bounds__(GEN_THREADS) k_gen(const GenArgs a) {
         __syncthreads();
         if (i0 == 0 && threadIdx.x == 0) atomicOr(&comp[0], 1u);   // 1 is not prime
 
-        // mark odd multiples of the base primes, starting at max(q^2, first in segment)
-        for (uint32_t b = warp; b < a.n_base; b += GEN_WARPS) {
-            const uint32_t q = __ldg(&a.base[b]);
-            if ((uint64_t)q * q > n_last) break;
-            if (q >= WARP_COOP_Q) break;
-            if (pre_ok && q <= PRE_MAX_Q) continue;          // in the pre-sieve
-            uint64_t start = (uint64_t)q * q;
-            if (start < n_first) {
-                const uint32_t rem = first_rem(n_first, q);
-                start = rem ? n_first + (q - rem) : n_first;
-                if ((start & 1) == 0) start += q;
+        // mark odd multiples of the base primes, starting at max(q^2, first in
+        // segment).  Small ones by a whole warp each; its lanes compute the starts
+        // of 32 of them at once
+        for (uint32_t b0 = 0; b0 < n_coop; b0 += 32 * GEN_WARPS) {
+            const uint32_t b = b0 + lane * GEN_WARPS + warp;
+            uint32_t q_l = 0, k_l = 0xffffffffu;
+            if (b < n_coop) {
+                q_l = __ldg(&a.base[b]);
+                const uint64_t sq = (uint64_t)q_l * q_l;
+                if (sq <= n_last && !(pre_ok && q_l <= PRE_MAX_Q)) {
+                    if (sq >= n_first) {
+                        k_l = (uint32_t)((sq - n_first) >> 1);
+                    } else {
+                        const uint32_t r = first_rem(i0, q_l);
+                        k_l = (q_l >> 1) >= r ? (q_l >> 1) - r : (q_l >> 1) + q_l - r;
+                    }
+                }
             }
-            for (uint64_t idx = (start - n_first) / 2 + (uint64_t)lane * q; idx < len; idx += 32ull * q)
-                atomicOr(&comp[idx >> 5], 1u << (idx & 31));
+            const uint32_t n_b = min(32u, (n_coop - b0 + GEN_WARPS - 1) / GEN_WARPS);
+            for (uint32_t t = 0; t < n_b; t++) {
+                const uint32_t q = __shfl_sync(0xffffffffu, q_l, t), k = __shfl_sync(0xffffffffu, k_l, t);
+                if (k >= len) continue;
+                for (uint32_t idx = k + lane * q; idx < len; idx += 32 * q)
+                    atomicOr(&comp[idx >> 5], 1u << (idx & 31));
+            }
         }
         // large base primes: one per thread (at most SEG / q + 1 marks each)
         {
-            for (uint32_t b = big0 + threadIdx.x; b < a.n_base; b += GEN_THREADS) {
+            const float fi0 = (float)(uint32_t)(i0 >> 20) * 1048576.0f + (float)(uint32_t)(i0 & 0xfffffu);
+            for (uint32_t b = n_coop + threadIdx.x; b < a.n_base; b += GEN_THREADS) {
                 const uint32_t q = __ldg(&a.base[b]);
-                if ((uint64_t)q * q > n_last) break;
-                uint64_t start = (uint64_t)q * q;
-                if (start < n_first) {
-                    const uint32_t rem = first_rem(n_first, q);
-                    start = rem ? n_first + (q - rem) : n_first;
-                    if ((start & 1) == 0) start += q;
-                }
-                for (uint64_t idx = (start - n_first) / 2; idx < len; idx += q)
+                const uint64_t sq = (uint64_t)q * q;
+                if (sq > n_last) break;
+                const uint64_t k = sq >= n_first ? (sq - n_first) >> 1 : first_multiple(i0, fi0, q);
+                if (k >= len) continue;
+                for (uint32_t idx = (uint32_t)k; idx < len; idx += q)
                     atomicOr(&comp[idx >> 5], 1u << (idx & 31));
             }
         }
         __syncthreads();
 
-        // extract: each warp owns a contiguous run of words
+        // extract: each warp owns a contiguous run of words.  The segment's output
+        // entries are taken with one atomic (one per 32 primes, all on the one
+        // counter, stalled the warps on its latency)
         const uint32_t wpw = seg_words / GEN_WARPS;
+        uint32_t cnt = 0;
+        for (uint32_t w = warp * wpw + lane; w < (warp + 1) * wpw; w += 32) cnt += __popc(~comp[w]);
+        cnt = __reduce_add_sync(0xffffffffu, cnt);
+        if (lane == 0) warp_n[warp] = cnt;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            uint32_t n = 0;
+            for (uint32_t w = 0; w < GEN_WARPS; w++) n += warp_n[w];
+            seg_base = n ? atomicAdd(a.count, (unsigned long long)n) : 0;
+        }
+        __syncthreads();
+        uint64_t slot = seg_base;
+        for (uint32_t w = 0; w < warp; w++) slot += warp_n[w];
+        const uint64_t part = 2 * (i0 + (uint64_t)warp * wpw * 32) + 1;    // the part's first number
         uint32_t qlen = 0;
-        for (uint32_t w0 = warp * wpw; w0 < (warp + 1) * wpw; w0 += BATCH) {
-            uint32_t w = w0 + lane;
-            uint32_t primes = lane < BATCH ? ~comp[w] : 0u;
-            uint32_t c = __popc(primes);
+        for (uint32_t w0 = 0; w0 < wpw; w0 += 32) {
+            const uint32_t w = w0 + lane;
+            uint32_t primes = w < wpw ? ~comp[warp * wpw + w] : 0u;
+            const uint32_t c = __popc(primes);
             uint32_t incl = c;
+#pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
                 uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
                 if (lane >= (unsigned)o) incl += t;
             }
-            uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
+            const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
             uint32_t pos = qlen + incl - c;
             while (primes) {
-                uint32_t bit = __ffs(primes) - 1;
+                queue[pos++] = (uint16_t)(w * 32 + __ffs(primes) - 1);
                 primes &= primes - 1;
-                queue[warp][pos++] = w * 32 + bit;
             }
             qlen += total;
             __syncwarp();
             uint32_t done = 0;
             while (qlen - done >= 32) {
-                uint32_t idx = queue[warp][done + lane];
-                emit<KIND>(a, 2 * (i0 + idx) + 1, true, lane);
+                emit<KIND>(a, part + 2 * queue[done + lane], true, slot + lane);
                 done += 32;
+                slot += 32;
             }
             __syncwarp();
             // move the remainder (< 32 entries) to the front
-            uint32_t rest = qlen - done;
-            uint32_t keep = lane < rest ? queue[warp][done + lane] : 0;
+            const uint32_t rest = qlen - done;
+            const uint16_t keep = lane < rest ? queue[done + lane] : (uint16_t)0;
             __syncwarp();
-            if (lane < rest) queue[warp][lane] = keep;
+            if (lane < rest) queue[lane] = keep;
             qlen = rest;
             __syncwarp();
         }
-        {
-            bool valid = lane < qlen;
-            uint32_t idx = valid ? queue[warp][lane] : 0;
-            emit<KIND>(a, 2 * (i0 + idx) + 1, valid, lane);
-        }
+        if (lane < qlen) emit<KIND>(a, part + 2 * queue[lane], true, slot + lane);
         __syncthreads();
     }
 }
 
-// CTAs of k_gen<KIND> resident at once on the device (occupancy API, once per kind)
+constexpr size_t GEN_SMEM = (SEG_WORDS + PRE_WORDS) * 4 + GEN_WARPS * QCAP * 2;
+
+// CTAs of k_gen<KIND> resident at once on the current device, whose shared-memory
+// limit for the kernel is raised on the first call (once per kind and device)
 template <int KIND>
 int gen_resident() {
-    static std::atomic<int> cached{0};
-    int n = cached.load(std::memory_order_relaxed);
+    static std::atomic<int> cached[64];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) dev = 0;
+    int n = cached[dev].load(std::memory_order_relaxed);
     if (n == 0) {
         int per_sm = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_gen<KIND>, GEN_THREADS, 0) != cudaSuccess ||
+        cudaFuncSetAttribute(k_gen<KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GEN_SMEM);
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_gen<KIND>, GEN_THREADS, GEN_SMEM) != cudaSuccess ||
             per_sm <= 0)
-            per_sm = CS_GEN_GRID_PER_SM;
+            per_sm = 1;
         n = sm_count() * per_sm;
-        cached.store(n, std::memory_order_relaxed);
+        cached[dev].store(n, std::memory_order_relaxed);
     }
     return n;
 }
@@ -438,7 +477,6 @@ GenArgs make_args(uint64_t lo, uint64_t hi, const uint32_t *base, uint32_t n_bas
     a.i_end = (hi + 1) / 2;
     const uint64_t odds = a.i_end > a.i_begin ? a.i_end - a.i_begin : 0;
     uint32_t seg = SEG_MIN;
-#if CS_GEN_ONE_WAVE
     // segment size: the range split evenly over whole waves of the resident
     // CTAs (k segments each), in multiples of SEG_MIN within [SEG_MIN, SEG], so
     // that no CTA waits on a partly filled last wave
@@ -449,13 +487,6 @@ GenArgs make_args(uint64_t lo, uint64_t hi, const uint32_t *base, uint32_t n_bas
         const uint64_t sz = (per + SEG_MIN - 1) / SEG_MIN * SEG_MIN;
         seg = (uint32_t)(sz < SEG_MIN ? SEG_MIN : (sz > SEG ? SEG : sz));
     }
-#else
-    // segment size: enough segments for every CTA of the grid to get
-    // CS_GEN_SEGS_PER_CTA of them, within [SEG_MIN, SEG]
-    uint64_t want = odds / ((uint64_t)sm_count() * CS_GEN_GRID_PER_SM * CS_GEN_SEGS_PER_CTA);
-    while (seg < SEG && seg < want) seg *= 2;
-    (void)resident;
-#endif
     a.seg = seg;
     a.n_seg = odds ? (odds + seg - 1) / seg : 0;
     a.emit_two = lo < 2 && hi >= 2;
@@ -463,12 +494,7 @@ GenArgs make_args(uint64_t lo, uint64_t hi, const uint32_t *base, uint32_t n_bas
 }
 
 int gen_grid(uint64_t n_seg, int resident) {
-#if CS_GEN_ONE_WAVE
     uint64_t g = (uint64_t)(resident > 0 ? resident : 1);
-#else
-    uint64_t g = (uint64_t)sm_count() * CS_GEN_GRID_PER_SM;
-    (void)resident;
-#endif
     if (n_seg < g) g = n_seg;
     return (int)(g ? g : 1);
 }
@@ -506,7 +532,7 @@ cudaError_t launch_gen_small(const DevPlan &pl, uint64_t lo, uint64_t hi, const 
     a.kch32 = pl.kch32; a.n_kch32 = pl.n_kch32;
     a.M_start = pl.M_start; a.SL = pl.SL;
     a.o0 = out; a.cap = cap; a.count = count; a.err = pl.stats + ST_ERROR;
-    k_gen<KIND_SMALL><<<gen_grid(a.n_seg, res), GEN_THREADS, 0, stream>>>(a);
+    k_gen<KIND_SMALL><<<gen_grid(a.n_seg, res), GEN_THREADS, GEN_SMEM, stream>>>(a);
     return cudaGetLastError();
 }
 
@@ -523,7 +549,7 @@ cudaError_t launch_gen_large(const DevPlan &pl, bool narrow, uint64_t lo, uint64
     a.o0 = p_out; a.o1 = r_out; a.o2 = v_out;
     a.cap = cap; a.count = count; a.err = pl.stats + ST_ERROR;
     if (narrow) {
-        k_gen<KIND_LARGE32><<<gen_grid(a.n_seg, res), GEN_THREADS, 0, stream>>>(a);
+        k_gen<KIND_LARGE32><<<gen_grid(a.n_seg, res), GEN_THREADS, GEN_SMEM, stream>>>(a);
     } else {
         // residues of the primes written: one wave of resident CTAs over the count
         static std::atomic<int> res_per_sm{0};
@@ -534,7 +560,7 @@ cudaError_t launch_gen_large(const DevPlan &pl, bool narrow, uint64_t lo, uint64
                 per_sm = 4;
             res_per_sm.store(per_sm, std::memory_order_relaxed);
         }
-        k_gen<KIND_LARGE64><<<gen_grid(a.n_seg, res), GEN_THREADS, 0, stream>>>(a);
+        k_gen<KIND_LARGE64><<<gen_grid(a.n_seg, res), GEN_THREADS, GEN_SMEM, stream>>>(a);
         k_large_res<<<sm_count() * per_sm, RES_THREADS, 0, stream>>>(a);
     }
     return cudaGetLastError();
@@ -551,9 +577,9 @@ cudaError_t launch_gen_pr(const DevPlan &kp, bool narrow, uint64_t lo, uint64_t 
     a.o0 = p_out; a.o1 = r_out;
     a.cap = cap; a.count = count; a.err = err;
     if (narrow)
-        k_gen<KIND_PR32><<<gen_grid(a.n_seg, res), GEN_THREADS, 0, stream>>>(a);
+        k_gen<KIND_PR32><<<gen_grid(a.n_seg, res), GEN_THREADS, GEN_SMEM, stream>>>(a);
     else
-        k_gen<KIND_PR64><<<gen_grid(a.n_seg, res), GEN_THREADS, 0, stream>>>(a);
+        k_gen<KIND_PR64><<<gen_grid(a.n_seg, res), GEN_THREADS, GEN_SMEM, stream>>>(a);
     return cudaGetLastError();
 }
 
@@ -564,7 +590,7 @@ cudaError_t launch_gen_list(uint64_t lo, uint64_t hi, const uint32_t *base, uint
     GenArgs a = make_args(lo, hi, base, n_base, res);
     if (a.n_seg == 0 && !a.emit_two) return cudaSuccess;
     a.o0 = out; a.cap = cap; a.count = count; a.err = err;
-    k_gen<KIND_LIST><<<gen_grid(a.n_seg, res), GEN_THREADS, 0, stream>>>(a);
+    k_gen<KIND_LIST><<<gen_grid(a.n_seg, res), GEN_THREADS, GEN_SMEM, stream>>>(a);
     return cudaGetLastError();
 }
 
