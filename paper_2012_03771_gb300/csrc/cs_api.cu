@@ -335,12 +335,11 @@ cs_status build_plan(cs_plan_s *pl, uint32_t P, uint64_t d, uint64_t M_start, ui
     if (const char *fa = getenv("CS_FAIL_ALLOC_AT")) pl->fail_alloc_at = strtoull(fa, nullptr, 10);
     pl->wheel = !pl->tune.no_wheel;
 
-    // K as 32- and 64-bit factor words; K itself when it fits in 64 bits
-    std::vector<uint32_t> kch32;
-    std::vector<uint64_t> kch64;
-    k_factor_words(qK, kch32, kch64);
-    bool k_fits = kch64.size() <= 1;
-    uint64_t K64 = kch64.empty() ? 1 : kch64[0];
+    // K as 32-bit factor words and as limbs; K itself when it fits in 64 bits
+    std::vector<uint32_t> kch32, klimb;
+    k_words(qK, kch32, klimb);
+    bool k_fits = klimb.size() <= 2;
+    uint64_t K64 = klimb[0] + (klimb.size() == 2 ? (uint64_t)klimb[1] << 32 : 0);
     if (k_fits) {
         unsigned __int128 lo = (unsigned __int128)M_start * K64;
         if (lo < (unsigned __int128)SL + 2) return fail(CS_EINVAL, "need M_start*K - SL >= 2");
@@ -658,9 +657,9 @@ cs_status build_plan(cs_plan_s *pl, uint32_t P, uint64_t d, uint64_t M_start, ui
     cs_status s;
     // the read-only tables go up together (one allocation, one copy)
     pl->stage(&dp.kch32, kch32);
-    pl->stage(&dp.kch64, kch64);
+    pl->stage(&dp.klimb, klimb);
     dp.n_kch32 = (uint32_t)kch32.size();
-    dp.n_kch64 = (uint32_t)kch64.size();
+    dp.n_klimb = (uint32_t)klimb.size();
     pl->stage(&dp.col_mask, col_mask);
     pl->stage(&dp.col_prefix, col_prefix);
     pl->stage(&dp.raw_of_col, raw_of_col);
@@ -786,8 +785,10 @@ struct Prof {
 
 namespace cs {
 
-void k_factor_words(const std::vector<uint32_t> &qK, std::vector<uint32_t> &w32, std::vector<uint64_t> &w64) {
+void k_words(const std::vector<uint32_t> &qK, std::vector<uint32_t> &w32, std::vector<uint32_t> &limbs) {
+    std::vector<uint64_t> w64;
     pack_k_words(qK, w32, w64);
+    limbs = k_limbs(w64);
 }
 
 
@@ -1186,25 +1187,22 @@ cs_status cs_k_mod_p(uint32_t P, uint64_t d, const uint64_t *p, uint64_t n, uint
     if (d == 0 || P > MAX_P) return fail(CS_EINVAL, "bad P or d");
     std::vector<uint32_t> qK, qd;
     if (!split_primes(P, d, qK, qd)) return fail(CS_EINVAL, "d must be squarefree and divide P#");
-    std::vector<uint32_t> kch32;
-    std::vector<uint64_t> kch64;
-    k_factor_words(qK, kch32, kch64);
+    std::vector<uint32_t> kch32, klimb;
+    k_words(qK, kch32, klimb);
     cudaStream_t st = (cudaStream_t)stream;
-    uint32_t *d32 = nullptr;
-    uint64_t *d64 = nullptr;
+    uint32_t *d32 = nullptr, *dl = nullptr;
     CS_CUDA(cudaMalloc(&d32, std::max<size_t>(kch32.size(), 1) * 4));
-    cudaError_t e = cudaMalloc(&d64, std::max<size_t>(kch64.size(), 1) * 8);
+    cudaError_t e = cudaMalloc(&dl, klimb.size() * 4);
     if (e == cudaSuccess && !kch32.empty())
         e = cudaMemcpyAsync(d32, kch32.data(), kch32.size() * 4, cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess && !kch64.empty())
-        e = cudaMemcpyAsync(d64, kch64.data(), kch64.size() * 8, cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(dl, klimb.data(), klimb.size() * 4, cudaMemcpyHostToDevice, st);
     DevPlan dp{};
     dp.kch32 = d32; dp.n_kch32 = (uint32_t)kch32.size();
-    dp.kch64 = d64; dp.n_kch64 = (uint32_t)kch64.size();
+    dp.klimb = dl; dp.n_klimb = (uint32_t)klimb.size();
     if (e == cudaSuccess) e = launch_kmodp(dp, p, n, r, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     cudaFree(d32);
-    cudaFree(d64);
+    cudaFree(dl);
     if (e != cudaSuccess) return cuda_fail(e, "cs_k_mod_p");
     return CS_OK;
 }

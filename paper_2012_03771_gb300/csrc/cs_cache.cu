@@ -22,7 +22,7 @@ using namespace cs;
 struct cs_cache_s {
     uint32_t P = 0;
     uint64_t d = 0, L_max = 0;
-    DevPlan kp{};                      // only kch32 / kch64 are used
+    DevPlan kp{};                      // only kch32 / klimb are used
     std::vector<void *> allocs;
     uint32_t *base = nullptr;          // odd primes <= sqrt(L_max), ascending
     uint32_t n_base = 0;
@@ -178,27 +178,26 @@ cs_status cache_new(uint32_t P, uint64_t d, uint64_t L_max, cs_cache_t *out) {
         }
     }
     if (rest != 1) return set_error(CS_EINVAL, "d must be squarefree and divide P#");
-    std::vector<uint32_t> kch32;
-    std::vector<uint64_t> kch64;
-    k_factor_words(qK, kch32, kch64);
+    std::vector<uint32_t> kch32, klimb;
+    k_words(qK, kch32, klimb);
 
     cs_cache_s *c = new (std::nothrow) cs_cache_s();
     if (!c) return set_error(CS_ENOMEM, "host allocation failed");
     c->P = P;
     c->d = d;
     cs_status s = CS_OK;
-    void *k32, *k64, *err;
+    void *k32, *kl, *err;
     if (!s) s = c->alloc(&k32, kch32.size() * 4);
-    if (!s) s = c->alloc(&k64, kch64.size() * 8);
+    if (!s) s = c->alloc(&kl, klimb.size() * 4);
     if (!s) s = c->alloc(&err, 8);
     if (!s && !kch32.empty()) s = cuda_err(upload_now(k32, kch32.data(), kch32.size() * 4), "upload");
-    if (!s && !kch64.empty()) s = cuda_err(upload_now(k64, kch64.data(), kch64.size() * 8), "upload");
+    if (!s) s = cuda_err(upload_now(kl, klimb.data(), klimb.size() * 4), "upload");
     if (!s) s = cuda_err(upload_now(err, nullptr, 8), "memset");
     if (s) { delete c; return s; }
     c->kp.kch32 = static_cast<uint32_t *>(k32);
     c->kp.n_kch32 = (uint32_t)kch32.size();
-    c->kp.kch64 = static_cast<uint64_t *>(k64);
-    c->kp.n_kch64 = (uint32_t)kch64.size();
+    c->kp.klimb = static_cast<uint32_t *>(kl);
+    c->kp.n_klimb = (uint32_t)klimb.size();
     c->err = static_cast<unsigned long long *>(err);
     s = cache_extend(c, std::max<uint64_t>(L_max, 2));
     if (s) { delete c; return s; }

@@ -47,11 +47,11 @@ struct DevPlan {
     uint64_t d;                   // K = P# / d
     int small_n;                  // N + x may equal a sieving prime or a prime of d
     uint64_t K64;                 // K when it fits in 64 bits (small_n only)
-    // K's prime factors packed into words: products below 2^31 / 2^64
+    // K's prime factors packed into words below 2^31, and K's 32-bit limbs
     const uint32_t *kch32;
     uint32_t n_kch32;
-    const uint64_t *kch64;
-    uint32_t n_kch64;
+    const uint32_t *klimb;
+    uint32_t n_klimb;
     // columns
     const uint32_t *col_mask;     // S32 words: bit z set iff raw offset z = x + SL is stored
     const uint32_t *col_prefix;   // S32 words: stored columns before word
@@ -105,7 +105,7 @@ cudaError_t launch_gen_large(const DevPlan &pl, bool narrow, uint64_t lo, uint64
                              const uint32_t *base, uint32_t n_base, void *p_out, void *r_out,
                              void *v_out, uint64_t cap, unsigned long long *count,
                              cudaStream_t stream);
-// Primes p in (lo, hi] with r = K mod p for the K of kp (kch32/kch64 only),
+// Primes p in (lo, hi] with r = K mod p for the K of kp (kch32/klimb only),
 // for a residue cache; narrow: 32-bit fields (hi < 2^30).
 cudaError_t launch_gen_pr(const DevPlan &kp, bool narrow, uint64_t lo, uint64_t hi, const uint32_t *base,
                           uint32_t n_base, void *p_out, void *r_out, uint64_t cap,
@@ -194,9 +194,9 @@ uint64_t walk_jobs_launches(const WalkJobs *wj);
 void walk_jobs_destroy(WalkJobs *wj);
 
 // K's prime factors qK packed into factor words below 2^31 (the generator's
-// lazily reduced Montgomery product) and below 2^64, first fit with the
-// largest factors first: K = product of either list.
-void k_factor_words(const std::vector<uint32_t> &qK, std::vector<uint32_t> &w32, std::vector<uint64_t> &w64);
+// lazily reduced Montgomery product), first fit with the largest factors first,
+// and K's 32-bit limbs, lowest first.
+void k_words(const std::vector<uint32_t> &qK, std::vector<uint32_t> &w32, std::vector<uint32_t> &limbs);
 
 // batch of G solves (tests of the solver)
 cudaError_t launch_modsolve(const uint64_t *p, const uint64_t *K, const uint64_t *L,

@@ -22,6 +22,7 @@
 
 #include "cs_arith.cuh"
 #include "cs_internal.h"
+#include "cs_residue.cuh"
 
 namespace cs {
 
@@ -50,9 +51,10 @@ constexpr uint32_t QCAP = 576;
 static_assert(SEG / GEN_WARPS <= 65536, "16-bit positions");
 static_assert(SEG_MIN % (32 * GEN_WARPS) == 0, "whole words per warp");
 
-// SMALL: tile records; LARGE32/64: (p, r, v0) of one plan; LIST: p only;
-// PR32/64: (p, r) for a residue cache shared by plans with the same K
-enum Kind { KIND_SMALL = 0, KIND_LARGE32 = 1, KIND_LARGE64 = 2, KIND_LIST = 3, KIND_PR32 = 4, KIND_PR64 = 5 };
+// SMALL: tile records; LARGE32: (p, r, v0) of one plan; LIST: 64-bit p only (the
+// residue kernel adds r and v0 for a plan, r for a cache); PR32: (p, r) for a
+// residue cache shared by plans with the same K
+enum Kind { KIND_SMALL = 0, KIND_LARGE32 = 1, KIND_LIST = 2, KIND_PR32 = 3 };
 
 struct GenArgs {
     uint64_t i_begin, i_end;      // odd indices [i_begin, i_end): numbers 2i+1
@@ -64,8 +66,8 @@ struct GenArgs {
     // residue parameters
     const uint32_t *kch32;
     uint32_t n_kch32;
-    const uint64_t *kch64;
-    uint32_t n_kch64;
+    const uint32_t *klimb;
+    uint32_t n_klimb;
     uint64_t M_start;
     uint32_t SL;
     // outputs
@@ -96,22 +98,12 @@ __device__ __forceinline__ uint32_t kmodp32(uint32_t p, uint32_t pinv, uint32_t 
     return acc >= p ? acc - p : acc;
 }
 
-// K mod p for 64-bit p from R^2 mod p: the product of the n factor words
-// starts at R^n mod p, which cancels their n factors R^-1
-__device__ __forceinline__ uint64_t kmodp64(uint64_t p, uint64_t pinv, uint64_t r2,
-                                            const uint64_t *kch, uint32_t n) {
-    if (n == 0) return 1ull % p;
-    uint64_t acc = mont64_rpow2(n, r2, p, pinv);
-    for (uint32_t i = 0; i < n; i++) acc = mont64_mul(acc, __ldg(&kch[i]), p, pinv);
-    return acc;
-}
-
 // slot: the output entry of this lane's prime
 template <int KIND>
 __device__ __forceinline__ void emit(const GenArgs &a, uint64_t p, bool valid, uint64_t slot) {
     // residue work for this lane's prime
     uint32_t e0 = 0, e1 = 0, e2 = 0, e3 = 0;
-    uint64_t w0 = 0, w1 = 0;
+    uint64_t w0 = 0;
     if (valid) {
         if (KIND == KIND_SMALL) {
             uint32_t p32 = (uint32_t)p;
@@ -135,18 +127,12 @@ __device__ __forceinline__ void emit(const GenArgs &a, uint64_t p, bool valid, u
             uint32_t r = kmodp32(p32, pinv, r1, r2, a.kch32, a.n_kch32);
             uint32_t rt = mont32_mul(r, r2, p32, pinv);
             e0 = p32; e1 = r; e2 = mont32_affine(rt, a.M_start, a.SL, r2, p32, pinv);   // SL < p
-        } else if (KIND == KIND_LARGE64) {
-            w0 = p;                                               // residues: k_large_res
         } else if (KIND == KIND_PR32) {
             uint32_t p32 = (uint32_t)p;
             uint32_t pinv = mont32_neg_inv(p32);
             e0 = p32;
             const uint32_t r2 = mont32_r2_fast(p32);
             e1 = kmodp32(p32, pinv, mont32_mul(r2, 1u, p32, pinv), r2, a.kch32, a.n_kch32);
-        } else if (KIND == KIND_PR64) {
-            uint64_t pinv = mont64_neg_inv(p);
-            w0 = p;
-            w1 = kmodp64(p, pinv, mont64_r2_fast(p, rcp_rn(u64_to_f(p))), a.kch64, a.n_kch64);
         } else {
             w0 = p;
         }
@@ -162,77 +148,69 @@ __device__ __forceinline__ void emit(const GenArgs &a, uint64_t p, bool valid, u
         reinterpret_cast<uint32_t *>(a.o0)[slot] = e0;
         reinterpret_cast<uint32_t *>(a.o1)[slot] = e1;
         reinterpret_cast<uint32_t *>(a.o2)[slot] = e2;
-    } else if (KIND == KIND_LARGE64) {
-        reinterpret_cast<uint64_t *>(a.o0)[slot] = w0;
     } else if (KIND == KIND_PR32) {
         reinterpret_cast<uint32_t *>(a.o0)[slot] = e0;
         reinterpret_cast<uint32_t *>(a.o1)[slot] = e1;
-    } else if (KIND == KIND_PR64) {
-        reinterpret_cast<uint64_t *>(a.o0)[slot] = w0;
-        reinterpret_cast<uint64_t *>(a.o1)[slot] = w1;
     } else {
         reinterpret_cast<uint64_t *>(a.o0)[slot] = w0;
     }
 }
 
-// Residues of the 64-bit large primes the generator wrote (o0): r = K mod p
-// (Section 3.1) into o1 and v = (r M_start + SL) mod p into o2, RES_ILP primes
-// per thread, every resident warp on the chains of 64-bit Montgomery products
-// (9% faster than inside the sieve kernel on L = 1e11).  The 32-bit residues stay in
+// Residues of the 64-bit primes the generator wrote (o0): r = K mod p (Section
+// 3.1) into o1 and, for a plan, v = (r M_start + SL) mod p into o2.  RES_ILP
+// primes per thread share the loads of K's limbs.  The 32-bit residues stay in
 // the sieve kernel, where they fill issue slots that its barriers and marking
-// phases leave idle (split out, the generator took 3.06 instead of 2.57 ms per
-// sieve on L = 1e9).
+// phases leave idle.
+//
+// Bound: the wide multiplies (a 32 x 32 + 64-bit one takes a scheduler about
+// five cycles, against one for an addition), two per limb and prime, one for p <
+// 2^32.  K = 1019#/210 (44 limbs) at p = 5e10: 34 ps per prime (60 as 64-bit
+// Montgomery products over 23 factor words), K = 1511#/210 (66 limbs) 43 (78), p <
+// 2^32: 26 and 32.  One prime per thread: 40, three: 36 (44 limbs).
 constexpr uint32_t RES_THREADS = 256;
-// primes per thread, whose Montgomery chains interleave (each chain is a
-// sequence of dependent multiplications, so one chain alone leaves issue slots
-// idle between them); on L = 1e11, generation and residues took 441 ms with
-// one, 420 with two, 426 with three and 427 with four (the wide multiplies'
-// pipe is then about 80% busy)
-#ifndef CS_RES_ILP
-#define CS_RES_ILP 2
-#endif
-constexpr int RES_ILP = CS_RES_ILP;
+constexpr int RES_ILP = 2;
+template <bool P32>
+__device__ __forceinline__ uint64_t res_k_mod_p(const ResMod &q, const uint32_t *limb, uint32_t n) {
+    // a modulus whose low word is too near 2^32 for the chain's products
+    if (q.p0 > RES_P0_MAX) {
+        uint64_t s = 0;
+        for (uint32_t i = 0; i < n; i++) s = res_step<P32>(s + __ldg(limb + i), q);
+        return res_finish<P32>(s, n, q);
+    }
+    uint64_t t = __ldg(limb);
+    for (uint32_t i = 1; i < n; i++) t = res_limb<P32>(t, __ldg(limb + i), q);
+    return res_finish<P32>(res_limb<P32>(t, 0, q), n, q);
+}
+template <bool P32, bool V>
 __global__ void __launch_bounds__(RES_THREADS) k_large_res(const GenArgs a) {
     const uint64_t n = min((uint64_t)*a.count, a.cap);
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
     const uint64_t *P = reinterpret_cast<const uint64_t *>(a.o0);
+    const uint32_t nl = a.n_klimb;
     for (uint64_t i0 = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i0 < n; i0 += RES_ILP * stride) {
-        uint64_t p[RES_ILP], pinv[RES_ILP], r2[RES_ILP], acc[RES_ILP];
-        float fp[RES_ILP];
+        ResMod q[RES_ILP];
+        uint64_t t[RES_ILP];
+        const uint32_t first = __ldg(a.klimb);
 #pragma unroll
         for (int k = 0; k < RES_ILP; k++) {
             const uint64_t i = i0 + k * stride;
-            p[k] = i < n ? P[i] : P[i0];                     // the extra chains repeat a valid prime
-            pinv[k] = mont64_neg_inv(p[k]);
-            fp[k] = rcp_rn(u64_to_f(p[k]));
-            r2[k] = mont64_r2_fast(p[k], fp[k]);
+            q[k] = res_mod<P32>(i < n ? P[i] : P[i0]);       // the extra chains repeat a valid prime
+            t[k] = first;
         }
-        // K mod p: R^n from R^2, then the n factor words (the same control flow for every chain)
-        const uint32_t nw = a.n_kch64;
-        if (nw == 0) {
+#pragma unroll 4
+        for (uint32_t l = 1; l < nl; l++) {
+            const uint32_t w = __ldg(a.klimb + l);
 #pragma unroll
-            for (int k = 0; k < RES_ILP; k++) acc[k] = 1ull % p[k];
-        } else {
-#pragma unroll
-            for (int k = 0; k < RES_ILP; k++) acc[k] = mont64_rpow2(nw, r2[k], p[k], pinv[k]);
-            for (uint32_t w = 0; w < nw; w++) {
-                const uint64_t f = __ldg(&a.kch64[w]);
-#pragma unroll
-                for (int k = 0; k < RES_ILP; k++) acc[k] = mont64_mul(acc[k], f, p[k], pinv[k]);
-            }
+            for (int k = 0; k < RES_ILP; k++) t[k] = res_limb<P32>(t[k], w, q[k]);
         }
 #pragma unroll
         for (int k = 0; k < RES_ILP; k++) {
             const uint64_t i = i0 + k * stride;
-            const uint64_t rt = mont64_mul(acc[k], r2[k], p[k], pinv[k]);
-            // M_start < 2^40: below p, or a quotient below 2^20 for p >= 2^20
-            const uint64_t ms = a.M_start < p[k] ? a.M_start
-                              : p[k] >= (1ull << 20) ? mod_q20(a.M_start, p[k], fp[k]) : a.M_start % p[k];
-            const uint64_t v = mont64_mul(rt, ms, p[k], pinv[k]) + a.SL;
-            if (i < n) {
-                reinterpret_cast<uint64_t *>(a.o1)[i] = acc[k];
-                reinterpret_cast<uint64_t *>(a.o2)[i] = v >= p[k] ? v - p[k] : v;
-            }
+            if (i >= n) continue;
+            uint64_t r = res_finish<P32>(res_limb<P32>(t[k], 0, q[k]), nl, q[k]);
+            if (!P32 && q[k].p0 > RES_P0_MAX) r = res_k_mod_p<false>(q[k], a.klimb, nl);
+            reinterpret_cast<uint64_t *>(a.o1)[i] = r;
+            if (V) reinterpret_cast<uint64_t *>(a.o2)[i] = res_affine<P32>(r, a.M_start, a.SL, q[k]);
         }
     }
 }
@@ -536,51 +514,66 @@ cudaError_t launch_gen_small(const DevPlan &pl, uint64_t lo, uint64_t hi, const 
     return cudaGetLastError();
 }
 
+namespace {
+// residues of the primes a launch of k_gen<KIND_LIST> over (.., hi] writes: one wave
+// of resident CTAs over the count
+template <bool P32, bool V>
+cudaError_t launch_res_kernel(const GenArgs &a, cudaStream_t stream) {
+    static std::atomic<int> res_per_sm{0};
+    int per_sm = res_per_sm.load(std::memory_order_relaxed);
+    if (per_sm == 0) {
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_large_res<P32, V>, RES_THREADS, 0) != cudaSuccess ||
+            per_sm <= 0)
+            per_sm = 4;
+        res_per_sm.store(per_sm, std::memory_order_relaxed);
+    }
+    k_large_res<P32, V><<<sm_count() * per_sm, RES_THREADS, 0, stream>>>(a);
+    return cudaGetLastError();
+}
+cudaError_t launch_res(const GenArgs &a, uint64_t hi, bool with_v, cudaStream_t stream) {
+    if (hi >> 32) return with_v ? launch_res_kernel<false, true>(a, stream) : launch_res_kernel<false, false>(a, stream);
+    return with_v ? launch_res_kernel<true, true>(a, stream) : launch_res_kernel<true, false>(a, stream);
+}
+}  // namespace
+
 cudaError_t launch_gen_large(const DevPlan &pl, bool narrow, uint64_t lo, uint64_t hi,
                              const uint32_t *base, uint32_t n_base, void *p_out, void *r_out,
                              void *v_out, uint64_t cap, unsigned long long *count,
                              cudaStream_t stream) {
-    const int res = narrow ? gen_resident<KIND_LARGE32>() : gen_resident<KIND_LARGE64>();
+    const int res = narrow ? gen_resident<KIND_LARGE32>() : gen_resident<KIND_LIST>();
     GenArgs a = make_args(lo, hi, base, n_base, res);
     if (a.n_seg == 0 && !a.emit_two) return cudaSuccess;
     a.kch32 = pl.kch32; a.n_kch32 = pl.n_kch32;
-    a.kch64 = pl.kch64; a.n_kch64 = pl.n_kch64;
+    a.klimb = pl.klimb; a.n_klimb = pl.n_klimb;
     a.M_start = pl.M_start; a.SL = pl.SL;
     a.o0 = p_out; a.o1 = r_out; a.o2 = v_out;
     a.cap = cap; a.count = count; a.err = pl.stats + ST_ERROR;
     if (narrow) {
         k_gen<KIND_LARGE32><<<gen_grid(a.n_seg, res), GEN_THREADS, GEN_SMEM, stream>>>(a);
-    } else {
-        // residues of the primes written: one wave of resident CTAs over the count
-        static std::atomic<int> res_per_sm{0};
-        int per_sm = res_per_sm.load(std::memory_order_relaxed);
-        if (per_sm == 0) {
-            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_large_res, RES_THREADS, 0) != cudaSuccess ||
-                per_sm <= 0)
-                per_sm = 4;
-            res_per_sm.store(per_sm, std::memory_order_relaxed);
-        }
-        k_gen<KIND_LARGE64><<<gen_grid(a.n_seg, res), GEN_THREADS, GEN_SMEM, stream>>>(a);
-        k_large_res<<<sm_count() * per_sm, RES_THREADS, 0, stream>>>(a);
+        return cudaGetLastError();
     }
-    return cudaGetLastError();
+    k_gen<KIND_LIST><<<gen_grid(a.n_seg, res), GEN_THREADS, GEN_SMEM, stream>>>(a);
+    const cudaError_t e = cudaGetLastError();
+    return e != cudaSuccess ? e : launch_res(a, hi, true, stream);
 }
 
 cudaError_t launch_gen_pr(const DevPlan &kp, bool narrow, uint64_t lo, uint64_t hi, const uint32_t *base,
                           uint32_t n_base, void *p_out, void *r_out, uint64_t cap,
                           unsigned long long *count, unsigned long long *err, cudaStream_t stream) {
-    const int res = narrow ? gen_resident<KIND_PR32>() : gen_resident<KIND_PR64>();
+    const int res = narrow ? gen_resident<KIND_PR32>() : gen_resident<KIND_LIST>();
     GenArgs a = make_args(lo, hi, base, n_base, res);
     if (a.n_seg == 0 && !a.emit_two) return cudaSuccess;
     a.kch32 = kp.kch32; a.n_kch32 = kp.n_kch32;
-    a.kch64 = kp.kch64; a.n_kch64 = kp.n_kch64;
+    a.klimb = kp.klimb; a.n_klimb = kp.n_klimb;
     a.o0 = p_out; a.o1 = r_out;
     a.cap = cap; a.count = count; a.err = err;
-    if (narrow)
+    if (narrow) {
         k_gen<KIND_PR32><<<gen_grid(a.n_seg, res), GEN_THREADS, GEN_SMEM, stream>>>(a);
-    else
-        k_gen<KIND_PR64><<<gen_grid(a.n_seg, res), GEN_THREADS, GEN_SMEM, stream>>>(a);
-    return cudaGetLastError();
+        return cudaGetLastError();
+    }
+    k_gen<KIND_LIST><<<gen_grid(a.n_seg, res), GEN_THREADS, GEN_SMEM, stream>>>(a);
+    const cudaError_t e = cudaGetLastError();
+    return e != cudaSuccess ? e : launch_res(a, hi, false, stream);
 }
 
 cudaError_t launch_gen_list(uint64_t lo, uint64_t hi, const uint32_t *base, uint32_t n_base,
@@ -596,7 +589,7 @@ cudaError_t launch_gen_list(uint64_t lo, uint64_t hi, const uint32_t *base, uint
 
 namespace {
 __global__ void k_kmodp(const uint64_t *p, uint64_t n, uint64_t *r, const uint32_t *kch32,
-                        uint32_t n32, const uint64_t *kch64, uint32_t n64) {
+                        uint32_t n32, const uint32_t *klimb, uint32_t n_limb) {
     for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n;
          i += (uint64_t)gridDim.x * blockDim.x) {
         uint64_t q = p[i];
@@ -604,9 +597,10 @@ __global__ void k_kmodp(const uint64_t *p, uint64_t n, uint64_t *r, const uint32
             uint32_t q32 = (uint32_t)q;
             uint32_t pinv = mont32_neg_inv(q32);
             r[i] = kmodp32(q32, pinv, mont32_r1(q32), mont32_r2(q32), kch32, n32);
+        } else if (q >> 32) {
+            r[i] = res_k_mod_p<false>(res_mod<false>(q), klimb, n_limb);
         } else {
-            uint64_t pinv = mont64_neg_inv(q);
-            r[i] = kmodp64(q, pinv, mont64_r2_fast(q, rcp_rn(u64_to_f(q))), kch64, n64);
+            r[i] = res_k_mod_p<true>(res_mod<true>(q), klimb, n_limb);
         }
     }
 }
@@ -617,8 +611,8 @@ cudaError_t launch_kmodp(const DevPlan &pl, const uint64_t *p, uint64_t n, uint6
     if (n == 0) return cudaSuccess;
     uint64_t blocks = (n + 255) / 256;
     if (blocks > 65535) blocks = 65535;
-    k_kmodp<<<(unsigned)blocks, 256, 0, stream>>>(p, n, r, pl.kch32, pl.n_kch32, pl.kch64,
-                                                   pl.n_kch64);
+    k_kmodp<<<(unsigned)blocks, 256, 0, stream>>>(p, n, r, pl.kch32, pl.n_kch32, pl.klimb,
+                                                   pl.n_klimb);
     return cudaGetLastError();
 }
 
