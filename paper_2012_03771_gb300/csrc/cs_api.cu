@@ -505,7 +505,9 @@ cs_status build_plan(cs_plan_s *pl, uint32_t P, uint64_t d, uint64_t M_start, ui
         double hits = (double)M_inc * (double)S / (double)std::max<uint64_t>(lo, 1);
         const MClasses mc = classes_for(lo);
         hits *= (double)(mc.items ? 1 : mc.n) / (double)mc.Q;
-        double seg = std::min<double>(std::max(1.0, std::ceil(hits / HITS_PER_ITEM)), (double)std::max<uint64_t>(M_inc, 1));
+        // at most 2^30 m per segment: the walk's offsets and clamped steps fit 32 bits
+        const double fewest = M_inc > (1ull << 30) ? 2.0 : 1.0;
+        double seg = std::min<double>(std::max(fewest, std::ceil(hits / HITS_PER_ITEM)), (double)std::max<uint64_t>(M_inc, 1));
         return (uint32_t)std::min(seg, 65536.0);
     };
     auto add_chunk = [&](uint64_t lo, uint64_t hi) {
@@ -679,6 +681,26 @@ cs_status build_plan(cs_plan_s *pl, uint32_t P, uint64_t d, uint64_t M_start, ui
     pl->stage(&dp.qd_pat_off, woff);
     pl->stage(&dp.qd_pat, wpat);
     dp.n_qd = (uint32_t)wq.size();
+    {
+        // the walk's test whether the wheel leaves N + x
+        uint64_t W = 1;
+        for (uint32_t q : wq) {
+            if (q == 2) dp.wh_even = 1;
+            else if (q <= 11) W *= q;
+        }
+        std::vector<uint32_t> keep((W + 31) / 32, 0);
+        for (uint64_t k = 0; k < W; k++)
+            if (std::gcd(k, W) == 1) keep[k >> 5] |= 1u << (k & 31);
+        if (W > 1) {
+            uint64_t km = 1;
+            for (uint32_t q : qK) km = km * q % W;
+            dp.wh_W = (uint32_t)W;
+            dp.wh_K = (uint32_t)km;
+            dp.wh_c = (uint32_t)((M_start % W * km + W - SL % W) % W);
+            magic_of(dp.wh_W, dp.wh_magic, dp.wh_shift);
+        }
+        pl->stage(&dp.wh_mask, keep);
+    }
     dp.compact = pl->layout == 1;
     dp.n_cls = pl->n_cls;
     dp.cls0 = pl->cls0;

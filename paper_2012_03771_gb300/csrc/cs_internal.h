@@ -68,6 +68,12 @@ struct DevPlan {
     const uint32_t *qd_kmod;      // K mod q
     const uint32_t *qd_pat_off;   // offset of q's pattern table in qd_pat
     const uint32_t *qd_pat;       // pattern[k]: bits i < 32 with (k + i) % q == 0
+    // which N + x the wheel leaves (hits on the others need no clear): wh_even = 1
+    // when d is even (only even x can be left), and for the product wh_W of d's odd
+    // primes up to 11 (0: none, or no wheel) N + x mod wh_W = (m - M_start) wh_K +
+    // wh_c + z looked up in wh_mask
+    uint32_t wh_even, wh_W, wh_magic, wh_shift, wh_K, wh_c;
+    const uint32_t *wh_mask;
     // compact layout: per residue class of m mod d (ascending), the stored
     // columns are the literal ones the wheel does not clear
     int compact;
@@ -130,6 +136,17 @@ cudaError_t launch_tile(const DevPlan &pl, const TileConfig &tc, const SmallPrim
 cudaError_t prepare_tile(int max_dynamic_smem);
 // shared memory the tile kernel uses besides the tile itself
 size_t tile_stage_bytes();
+
+// multiplier and shift of the division by 2 <= W < 2^16 of numbers below 2^31
+inline void magic_of(uint32_t W, uint32_t &magic, uint32_t &shift) {
+    shift = 0;
+    while ((2u << shift) <= W) shift++;
+    magic = (uint32_t)(((1ull << (32 + shift)) + W - 1) / W);
+    if ((W & (W - 1)) == 0) {           // a power of two: 2^31 and one shift less
+        magic = 1u << 31;
+        shift--;
+    }
+}
 
 enum LargeMode { LARGE_PAPER = 1, LARGE_THREE_GAP = 2 };
 // m-classes of the three-gap walk: only m = c (mod Q) for the n classes c with

@@ -44,6 +44,7 @@ struct LargeArgs {
     // {first m - M_start (or NO_WALKER), v there, d_a, u_b} and {steps of m a, b}
     const uint4 *desc0;
     const uint2 *desc1;
+    uint32_t q_magic, q_shift;   // division by mc.Q (class items whose Q is d)
 };
 
 // v0 = (r * M_start + SL) mod p, for primes from a shared residue cache
@@ -73,90 +74,82 @@ struct Counters {
     unsigned long long solves = 0, levels = 0, err = 0;
 };
 
-// One hit of prime p at m = M_start + moff, raw offset z = x + SL = 2SL - v
-// for v = (r m + SL) mod p <= 2SL.  Branch-free up to the atomic: the row and
-// column tests are bit lookups in small tables (coprime-m mask, stored-x
-// mask, each interleaved with its per-word prefix counts) that stay in L1.
-// The prime is read (from the chunk's array, entry idx) only when N + x can be
-// a sieving prime itself (K below 2^64).
-// The fields of a plan that a hit reads, held in registers by the multi-job
-// walk (its plan descriptors sit in shared memory, which the walkers' queue
-// stores would otherwise make it reload at every hit); the one-chunk walk reads
-// them from its kernel parameters.
-struct HitView {
-    const uint2 *row_tab, *col_tab;
-    uint64_t *bits;
-    uint32_t wpr, SL;
-    int small_n, compact;
-    uint64_t M_start, K64;
-    const uint32_t *cls_word, *cmask, *cprefix;
-    uint32_t n_cls, S32;
-};
-__device__ __forceinline__ HitView hit_view(const DevPlan &p) {
-    return HitView{p.row_tab, p.col_tab, p.bits, p.wpr, p.SL, p.small_n, p.compact, p.M_start, p.K64,
-                   p.cls_word, p.cmask, p.cprefix, p.n_cls, p.S32};
+// Clears the bit of a stored column, or writes its record.  BKT: a record in this
+// CTA's region for its band of rows (slot from the CTA's per-band counter bkt_s in
+// shared memory, one plain store); a full region clears directly.
+template <bool BKT>
+__device__ __forceinline__ void clear_cell(const DevPlan &pl, uint32_t row, uint32_t col, uint32_t *bkt_s) {
+    if constexpr (BKT) {
+        const uint32_t band = row >> pl.band_log;
+        const uint32_t slot = atomicAdd(bkt_s + band, 1u);
+        if (slot < pl.region_cap) {
+            pl.bkt[((uint64_t)band * pl.n_regions + blockIdx.x) * pl.region_cap + slot] =
+                (row & ((1u << pl.band_log) - 1)) * (64 * pl.wpr) + col;
+            return;
+        }
+    }
+    // 32-bit view of the row's words: column col is bit (col mod 32) of word col >> 5
+    atomicAnd(reinterpret_cast<unsigned int *>(pl.bits) + (uint64_t)row * (2 * pl.wpr) + (col >> 5), ~bit_at(col));
 }
 
-// BKT: the stored hit becomes a record in this CTA's region for its band of
-// rows (slot from the CTA's per-band counter bkt_s in shared memory, one plain
-// store); a full region clears directly.
-// rt = row_tab[moff >> 5] {coprime-m mask, rows before}, ct = col_tab[z >> 5]
-// {stored-x mask, columns before}: loaded by the caller, the walk one step
-// ahead so that the loads are in flight while the previous hit is recorded.
-// ROWS: m is known to be a row, and its row index is row_in (rt unused; the
-// class-item walk with Q = d, literal layout).
-template <class UT, class PV = DevPlan, bool BKT = false, bool ROWS = false>
-__device__ __forceinline__ void record_hit_rc(const PV &pl, uint64_t moff, uint32_t z, uint2 rt, uint2 ct,
-                                              const UT *Pp, uint32_t idx, Counters &c, uint32_t *bkt_s = nullptr,
-                                              uint32_t row_in = 0) {
-    const uint32_t ms = (uint32_t)moff;                  // bit of m in its 32-m word: ms mod 32
-    // m coprime to d, x coprime to K
-    bool ok = ROWS ? bit_of(ct.x, z) != 0 : (bit_of(rt.x, ms) & bit_of(ct.x, z)) != 0;
+// floor(x / W) for x < 2^31 and 2 <= W < 2^16: umulhi by ceil(2^(32 + s) / W), s =
+// floor(log2 W), whose excess over 2^(32 + s) / W is below 1, shifts the quotient by
+// less than 2^31 / 2^(32 + s) < 1 / W.
+__device__ __forceinline__ uint32_t div_magic(uint32_t x, uint32_t magic, uint32_t shift) {
+    return __umulhi(x, magic) >> shift;
+}
+
+// Whether the wheel of d's primes leaves N + x: its bit is 0 already when a prime of
+// d divides N + x (the tile sieve writes it so, and a hit's N + x is no prime of d), so
+// such a hit is counted but not cleared.  Three quarters of the stored hits for
+// d = 210.  x odd for even d (K and the m of rows are odd then), then N + x mod the
+// product of d's odd primes up to 11.
+__device__ __forceinline__ bool wheel_leaves(const DevPlan &pl, uint32_t moff, uint32_t z) {
+    bool keep = ((z ^ pl.SL) & pl.wh_even) == 0;
+    if (pl.wh_W && keep) {
+        const uint32_t mr = moff - div_magic(moff, pl.wh_magic, pl.wh_shift) * pl.wh_W;
+        const uint32_t t = mr * pl.wh_K + pl.wh_c + z;           // below 1155^2 + 1155 + 2^21
+        const uint32_t r = t - div_magic(t, pl.wh_magic, pl.wh_shift) * pl.wh_W;
+        keep = bit_of(__ldg(&pl.wh_mask[r >> 5]), r) != 0;
+    }
+    return keep;
+}
+
+// One hit of prime p at m = M_start + moff, raw offset z = x + SL = 2SL - v for v = (r
+// m + SL) mod p <= 2SL, where x is a stored column.  ROWS: m is a row, of index
+// row_in (literal layout); otherwise the row table's word of m (rt: coprime-m mask and
+// rows before it) says so.  p is read (from the chunk's array, entry idx) only when
+// N + x can be a sieving prime itself (K below 2^64).
+template <class UT, bool BKT, bool ROWS>
+__device__ __forceinline__ void take_hit(const DevPlan &pl, uint32_t moff, uint32_t z, uint2 rt, const UT *Pp,
+                                         uint32_t idx, uint32_t &F, uint32_t *bkt_s, uint32_t row_in = 0) {
+    uint32_t row = row_in, row_below = 0;
+    bool ok = true;
+    if (!ROWS) {
+        row_below = __popc(bits_below(rt.x, moff));
+        row = rt.y + row_below;
+        ok = bit_of(rt.x, moff) != 0;
+    }
     if (pl.small_n) {
-        unsigned __int128 n = (unsigned __int128)(pl.M_start + moff) * pl.K64 + z - pl.SL;
+        const unsigned __int128 n = (unsigned __int128)(pl.M_start + moff) * pl.K64 + z - pl.SL;
         ok = ok && n != (unsigned __int128)Pp[idx];      // N + x is p itself
     }
-    const uint32_t row_below = ROWS ? 0u : __popc(bits_below(rt.x, ms));
-    const uint32_t row = ROWS ? row_in : rt.y + row_below;
-    uint32_t col = ct.y + __popc(bits_below(ct.x, z));
-    bool store = ok;                                     // F counts every stored x coprime to K
-    if (!ROWS && pl.compact && ok) {
+    F += ok;                                             // F counts every stored x coprime to K
+    if (!ok || !wheel_leaves(pl, moff, z)) return;
+    uint32_t col;
+    if (!ROWS && pl.compact) {
         // the row's class keeps only x with gcd(N + x, d) = 1; class of the
         // first row of this 32-m word, plus the rows before m in the word
         uint32_t cls = __ldg(&pl.cls_word[moff >> 5]) + row_below;
         while (cls >= pl.n_cls) cls -= pl.n_cls;
-        const uint32_t ccw = __ldg(&pl.cmask[(size_t)cls * pl.S32 + (z >> 5)]);
-        col = __ldg(&pl.cprefix[(size_t)cls * pl.S32 + (z >> 5)]) + __popc(bits_below(ccw, z));
-        store = bit_of(ccw, z) != 0;
+        const uint32_t w = __ldg(&pl.cmask[(size_t)cls * pl.S32 + (z >> 5)]);
+        if (!bit_of(w, z)) return;
+        col = __ldg(&pl.cprefix[(size_t)cls * pl.S32 + (z >> 5)]) + __popc(bits_below(w, z));
+    } else {
+        const uint2 ct = __ldg(&pl.col_tab[z >> 5]);
+        col = ct.y + __popc(bits_below(ct.x, z));
     }
-    // 32-bit view of the row's words: column col is bit (col mod 32) of word col >> 5
-    if (store) {
-        bool direct = true;
-        if constexpr (BKT) {
-            const uint32_t band = row >> pl.band_log;
-            const uint32_t slot = atomicAdd(bkt_s + band, 1u);
-            if (slot < pl.region_cap) {
-                pl.bkt[((uint64_t)band * pl.n_regions + blockIdx.x) * pl.region_cap + slot] =
-                    (row & ((1u << pl.band_log) - 1)) * (64 * pl.wpr) + col;
-                direct = false;
-            }
-        }
-        if (direct)
-            atomicAnd(reinterpret_cast<unsigned int *>(pl.bits) + (uint64_t)row * (2 * pl.wpr) + (col >> 5),
-                      ~bit_at(col));
-    }
-    c.F += ok;
-}
-template <class UT, class PV = DevPlan, bool BKT = false>
-__device__ __forceinline__ void record_hit_z(const PV &pl, uint64_t moff, uint32_t z, const UT *Pp,
-                                             uint32_t idx, Counters &c, uint32_t *bkt_s = nullptr) {
-    record_hit_rc<UT, PV, BKT>(pl, moff, z, __ldg(&pl.row_tab[moff >> 5]), __ldg(&pl.col_tab[z >> 5]), Pp, idx, c,
-                               bkt_s);
-}
-template <class UT>
-__device__ __forceinline__ void record_hit(const DevPlan &pl, uint64_t moff, UT v, const UT *Pp, uint32_t idx,
-                                           Counters &c) {
-    record_hit_z<UT>(pl, moff, 2 * pl.SL - (uint32_t)v, Pp, idx, c);
+    clear_cell<BKT>(pl, row, col, bkt_s);
 }
 
 template <class UT, class ST>
@@ -191,7 +184,10 @@ __global__ void __launch_bounds__(LARGE_THREADS) k_large(const LargeArgs a) {
             while (true) {
                 if (v <= w) {
                     c.hits++;
-                    record_hit<UT>(pl, m_lo + m, v, Pp, (uint32_t)i, c);
+                    const uint32_t z = 2 * pl.SL - (uint32_t)v;
+                    if (bit_of(__ldg(&pl.col_mask[z >> 5]), z))
+                        take_hit<UT, false, false>(pl, (uint32_t)(m_lo + m), z, __ldg(&pl.row_tab[(m_lo + m) >> 5]), Pp,
+                                                   (uint32_t)i, c.F, nullptr);
                     if (++m >= Mseg) break;
                     v += r;
                     if (v >= p) v -= p;
@@ -253,6 +249,20 @@ struct TGItem {
     MT ma, mb;                     // steps of m (clamped to M_inc)
 };
 
+// A warp's buffered hits {m - M_start, z}, at most 31 left over and four of each lane
+// from a pass, and (read only for K below 2^64) the chunk index of each hit's prime.
+constexpr int TG_UNROLL = 4;                        // steps of a pass
+struct HitBuf {
+    uint2 hit[31 + 32 * TG_UNROLL];
+    uint32_t idx[31 + 32 * TG_UNROLL];
+};
+// Class items of a launch: each class's residue of m - M_start, and for the rows'
+// indices (Q = d) the rank of every residue of m mod Q among the coprime ones.
+struct WalkClasses {
+    const uint8_t *item_off, *rank;
+    uint32_t ms, magic, shift, rank0;
+};
+
 // three-gap steps per lane between queue checks, class walkers (class items
 // and the two walkers mod 6): their m-segments hold nearly the same number of
 // hits (about the walked hits per item, 128), so the lanes of a warp finish
@@ -270,6 +280,7 @@ struct TGItem {
 #endif
 constexpr int TG_STEPS = CS_TG_STEPS;               // class walks (long walkers)
 constexpr int TG_STEPS_ALL_M = CS_TG_STEPS_ALL_M;   // one-walker items (the light chunks)
+static_assert(TG_STEPS % TG_UNROLL == 0 && TG_STEPS_ALL_M % TG_UNROLL == 0, "whole passes");
 constexpr int TG_WARPS = LARGE_THREADS / 32;
 
 // the same for k < 2^31 in one reduction (fr = rcp_rn(p) for 32-bit p)
@@ -299,19 +310,27 @@ __device__ __forceinline__ uint64_t mul_add_mod(uint64_t v, uint64_t r, uint32_t
 // then the warp's counters go to the plan's statistics.  item_off: the class
 // residues of class items (shared memory).
 // CI: 0 = m-class walkers, 1 = class items, 2 = class items mod Q = d in the
-// literal layout, whose rows follow from the walker's steps: every walked m is
-// a row, and a step of k Q in m passes k phi(Q) rows.
+// literal layout: every walked m is a row, whose index follows from m alone.
 // PRE: the walkers come prepared by k_tg_prep (one-walker items, one segment).
-template <class UT, class ST, class MT, int NC, int CI, bool JOBS = false, bool BKT = false, bool PRE = false>
-__device__ __forceinline__ void walk_warp(const LargeArgs &a, TGItem<MT> *q, const uint8_t *item_off,
-                                          uint64_t first, uint64_t n_warps, uint32_t *bkt_s = nullptr) {
+// col_mask: the stored-x mask's words, in shared memory (SM) or global.
+//
+// The lanes step together.  A step is two comparisons, four predicated additions
+// and one table word (is x stored?, loaded a step ahead); after a pass of four
+// steps, the lanes push the third of their visits that are stored (m, z) to the
+// warp's buffer.  Every 32 hits are taken at full lanes (take_hit: row, F, wheel,
+// column, clear), the row table's words of one group loading until the next one is
+// due.  Taking each hit where it is visited ran that longer path with a quarter of
+// the lanes and read the row table at every visit.
+template <class UT, class ST, class MT, int NC, int CI, bool SM, bool JOBS = false, bool BKT = false, bool PRE = false>
+__device__ __forceinline__ void walk_warp(const LargeArgs &a, TGItem<MT> *q, HitBuf &buf, const uint32_t *col_mask,
+                                          const WalkClasses &wc, uint64_t first, uint64_t n_warps,
+                                          uint32_t *bkt_s = nullptr) {
     static_assert(!CI || NC == 1, "class items walk one class per item");
     static_assert(!PRE || (NC == 1 && !CI && !JOBS), "prepared walkers: one-walker items");
+    const uint8_t *item_off = wc.item_off;
     constexpr int QCAP = 32 * (NC + 1);   // a refill adds at most 32 NC walkers
     const uint32_t n_cls_items = CI ? a.mc.items : 1;
     const DevPlan &pl = a.pl;
-    // the hit path's plan fields: kernel parameters, or registers for the multi-job walk
-    [[maybe_unused]] const HitView hv = JOBS ? hit_view(pl) : HitView{};
     const UT *Pp = reinterpret_cast<const UT *>(a.p);
     const UT *Rp = reinterpret_cast<const UT *>(a.r);
     const UT *Vp = reinterpret_cast<const UT *>(a.v);
@@ -324,28 +343,48 @@ __device__ __forceinline__ void walk_warp(const LargeArgs &a, TGItem<MT> *q, con
     const unsigned lane = threadIdx.x & 31;
     const unsigned lt_mask = (1u << lane) - 1;
     const uint64_t n_items = n * n_seg * n_cls_items;
-    // any step >= M ends a walker (its segment is at most M long); two clamped
-    // steps still add up below 2^32
-    const uint64_t cap_step = M;
+    // any step of a segment's length ends a walker; segments are at most 2^30 long
+    // (the plan splits longer m-ranges), so m and two clamped steps add up below 2^32
     const uint64_t seg_len = (M + n_seg - 1) / n_seg;
+    const uint64_t cap_step = seg_len;
     Counters c;
     if (M == 0) return;
 
     uint64_t batch = first;            // next batch of 32 items to prepare
     uint32_t qhead = 0, qcount = 0;    // warp-uniform ring state
-    bool active = false;
-    // walker: m offset, segment end, raw offset z = 2SL - v, and the three steps
-    // precomputed: down (v >= d_a, z <= 2SL - d_a): m += a, z += d_a; up
-    // (v <= 2SL - u_b, z >= u_b): m += b, z -= u_b; else m += a + b,
-    // z += d_a - u_b
-    MT moff = 0, end = 0, ma = 0, mb = 0, mab = 0;
-    uint32_t z = 0, idx = 0, da = 0, ub = 0, wmda = 0, nub = 0, dmu = 0;
-    // the current hit's row and column table words (loaded one step ahead)
-    const uint2 *row_tab = JOBS ? hv.row_tab : pl.row_tab;
-    const uint2 *col_tab = JOBS ? hv.col_tab : pl.col_tab;
-    uint2 rt = make_uint2(0, 0), ct = make_uint2(0, 0);
+    // walker: m offset and its segment's end (idle: moff >= end), raw offset z = 2SL -
+    // v, and the steps: z < u_b allows m += a, z += d_a; z > 2SL - d_a needs m += b, z -=
+    // u_b; between the two, both
+    MT moff = 0, end = 0, ma = 0, mb = 0;
+    uint32_t z = 0, da = 0, ub = 0, wmda = 0, idx = 0;
     constexpr bool ROWS = CI == 2;
-    uint32_t row = 0, ra = 0, rb = 0, rab = 0;   // ROWS: row of the current hit, rows per step
+    uint32_t n_buf = 0, n_due = 0;     // hits in the buffer, and in the group due (warp-uniform)
+    uint2 due = make_uint2(0, 0), due_rt = make_uint2(0, 0);   // the group due: this lane's hit, its row-table word
+    uint32_t due_idx = 0;
+    auto take_due = [&]() {
+        if (lane < n_due) {
+            uint32_t row = 0;
+            if constexpr (ROWS) {
+                const uint32_t m = due.x + wc.ms, k = div_magic(m, wc.magic, wc.shift);
+                row = k * n_cls_items + wc.rank[m - k * Q] - wc.rank0;
+            }
+            uint32_t F = 0;
+            take_hit<UT, BKT, ROWS>(pl, due.x, due.y, due_rt, Pp, due_idx, F, bkt_s, row);
+            if (!ROWS || pl.small_n) c.F += F;       // else counted at its visit
+        }
+    };
+    // makes the last n <= 32 buffered hits the group due
+    auto next_due = [&](uint32_t n) {
+        __syncwarp();
+        n_buf -= n;
+        n_due = n;
+        if (lane < n) {
+            due = buf.hit[n_buf + lane];
+            if (!ROWS) due_rt = __ldg(&pl.row_tab[due.x >> 5]);
+            if (pl.small_n) due_idx = buf.idx[n_buf + lane];
+        }
+        __syncwarp();
+    };
 
     while (true) {
         // refill: prepare 32 items when the queue can take their walkers
@@ -413,8 +452,10 @@ __device__ __forceinline__ void walk_warp(const LargeArgs &a, TGItem<MT> *q, con
                     dk[k] = 0;
                 }
                 if (ok && w == 0) {
-                    // SL = 0 (Q = 1, NC = 1): every p-th m; v stays 0
+                    // SL = 0 (Q = 1, NC = 1): every p-th m; v stays 0 (u_b = 1: z = 0
+                    // always takes the step down, of 0 in z and p in m)
                     ma_ = pp;
+                    ub_ = 1;
                     if (vv > w) {
                         UT t, y;
                         c.solves++;
@@ -487,67 +528,82 @@ __device__ __forceinline__ void walk_warp(const LargeArgs &a, TGItem<MT> *q, con
             __syncwarp();
         }
         // hand queued items to idle lanes
-        const unsigned idle = __ballot_sync(0xffffffffu, !active);
+        const unsigned idle = __ballot_sync(0xffffffffu, moff >= end);
         if (idle && qcount) {
             const uint32_t rank = __popc(idle & lt_mask);
-            const uint32_t take = min((uint32_t)__popc(idle), qcount);
-            if (!active && rank < take) {
+            const uint32_t n_take = min((uint32_t)__popc(idle), qcount);
+            if (moff >= end && rank < n_take) {
                 const TGItem<MT> e = q[(qhead + rank) % QCAP];
-                moff = e.moff; end = e.end; z = (uint32_t)w - e.v; idx = e.idx; da = e.da; ub = e.ub;
+                moff = e.moff; end = e.end; z = (uint32_t)w - e.v;
+                da = e.da; ub = e.ub;
                 ma = e.ma; mb = e.mb;
-                mab = ma + mb;                       // ma, mb <= M_inc < 2^31
                 wmda = (uint32_t)w - da;
-                nub = 0u - ub;
-                dmu = da - ub;                       // both wrap; z ends in [0, 2SL]
-                rt = __ldg(&row_tab[moff >> 5]);
-                ct = __ldg(&col_tab[z >> 5]);
-                if constexpr (ROWS) {
-                    // steps are multiples of Q (a clamped one ends the walker)
-                    row = rt.y + __popc(bits_below(rt.x, (uint32_t)moff));
-                    ra = (uint32_t)ma / Q * n_cls_items;
-                    rb = (uint32_t)mb / Q * n_cls_items;
-                    rab = ra + rb;
-                }
-                active = true;
+                idx = e.idx;
             }
-            qhead = (qhead + take) % QCAP;
-            qcount -= take;
+            qhead = (qhead + n_take) % QCAP;
+            qcount -= n_take;
             __syncwarp();
         }
-        const unsigned act = __ballot_sync(0xffffffffu, active);
-        if (!act) {
+        if (!__any_sync(0xffffffffu, moff < end)) {
             if (qcount == 0 && batch * 32 >= n_items) break;
             continue;
         }
-        // up to TG_STEPS three-distance steps per active lane between queue
-        // checks (each step as selects)
+        // up to TG_STEPS three-distance steps per active lane between queue checks
         constexpr int STEPS = NC == 1 && !CI ? TG_STEPS_ALL_M : TG_STEPS;
-        int u = 0;
-        for (; u < STEPS && active; u++) {
-            const bool down = z <= wmda;
-            const bool up = z >= ub;
-            const uint32_t zn = z + (down ? da : (up ? nub : dmu));
-            const MT step = down ? ma : (up ? mb : mab);
-            active = step < end - moff;
-            const MT mn = moff + step;
-            // the next hit's table words, in flight while this one is recorded
-            uint2 rtn = rt, ctn = ct;
-            if (active) {
-                if constexpr (!ROWS) rtn = __ldg(&row_tab[mn >> 5]);
-                ctn = __ldg(&col_tab[zn >> 5]);
+        uint32_t cw = SM ? col_mask[z >> 5] : __ldg(&col_mask[z >> 5]);
+#pragma unroll 1
+        for (int u = 0; u < STEPS; u += TG_UNROLL) {
+            bool push[TG_UNROLL];
+            uint2 at[TG_UNROLL];
+            uint32_t n_push = 0;
+#pragma unroll
+            for (int v = 0; v < TG_UNROLL; v++) {
+                // an idle lane stays where it is (z remains a valid offset)
+                const bool act = moff < end;
+                const bool down = act && z < ub, up = act && z > wmda;
+                uint32_t zn = z;
+                MT mn = moff;
+                if (down) zn += da, mn += ma;
+                if (up) zn -= ub, mn += mb;
+                const uint32_t cwn = SM ? col_mask[zn >> 5] : __ldg(&col_mask[zn >> 5]);
+                const bool ok = act && bit_of(cw, z);
+                c.hits += act;                       // one visited hit per step taken
+                push[v] = ok;
+                if constexpr (ROWS) {
+                    if (!pl.small_n) {
+                        // a row: counted here, and even N + x need no clear
+                        c.F += ok;
+                        push[v] = ok && ((z ^ pl.SL) & pl.wh_even) == 0;
+                    }
+                }
+                at[v] = make_uint2(moff, z);
+                n_push += push[v];
+                z = zn;
+                cw = cwn;
+                moff = mn;
             }
-            if constexpr (JOBS)
-                record_hit_rc<UT>(hv, (uint64_t)moff, z, rt, ct, Pp, idx, c);
-            else
-                record_hit_rc<UT, DevPlan, BKT, ROWS>(pl, (uint64_t)moff, z, rt, ct, Pp, idx, c, bkt_s, row);
-            if constexpr (ROWS) row += down ? ra : (up ? rb : rab);
-            rt = rtn;
-            ct = ctn;
-            z = zn;
-            moff = mn;
+            // the lanes' places in the buffer, from ballots of their counts' bits
+            const unsigned b0 = __ballot_sync(0xffffffffu, n_push & 1), b1 = __ballot_sync(0xffffffffu, n_push & 2),
+                           b2 = __ballot_sync(0xffffffffu, n_push & 4);
+            uint32_t slot = n_buf + __popc(b0 & lt_mask) + 2 * __popc(b1 & lt_mask) + 4 * __popc(b2 & lt_mask);
+#pragma unroll
+            for (int v = 0; v < TG_UNROLL; v++)
+                if (push[v]) {
+                    buf.hit[slot] = at[v];
+                    if (pl.small_n) buf.idx[slot] = idx;
+                    slot++;
+                }
+            n_buf += __popc(b0) + 2 * __popc(b1) + 4 * __popc(b2);
+            while (n_buf >= 32) {
+                take_due();
+                next_due(32);
+            }
+            if (!__any_sync(0xffffffffu, moff < end)) break;
         }
-        c.hits += u;                                 // one hit per step taken
     }
+    take_due();
+    next_due(n_buf);
+    take_due();
 
     const unsigned long long F = warp_sum(c.F), hits = warp_sum(c.hits);
     c.solves = warp_sum(c.solves);
@@ -562,26 +618,42 @@ __device__ __forceinline__ void walk_warp(const LargeArgs &a, TGItem<MT> *q, con
     }
 }
 
-template <class UT, class ST, class MT, int NC, int CI = 0, bool BKT = false, bool PRE = false>
+template <class UT, class ST, class MT, int NC, int CI, bool SM, bool BKT, bool PRE>
 __global__ void __launch_bounds__(LARGE_THREADS, sizeof(UT) == 4 ? CS_TG_MIN_BLOCKS : CS_TG_MIN_BLOCKS_WIDE) k_large_tg(const LargeArgs a) {
     constexpr int QCAP = 32 * (NC + 1);
     __shared__ TGItem<MT> queue[TG_WARPS][QCAP];
+    __shared__ HitBuf hits[TG_WARPS];
     __shared__ uint8_t item_off[CI ? MAX_CLASS_ITEMS : 1];   // class items: residue of each class
-    extern __shared__ uint32_t bkt_s[];                      // BKT: records in this CTA's region per band
+    __shared__ uint8_t rank[CI == 2 ? 256 : 1];
+    extern __shared__ uint32_t walk_smem[];                  // BKT: records in this CTA's region per band; SM: column mask
+    uint32_t *bkt_s = walk_smem, *mask_s = walk_smem + (BKT ? a.pl.n_bands : 0);
     const DevPlan &pl = a.pl;
+    WalkClasses wc{item_off, rank, 0, a.q_magic, a.q_shift, 0};
     if constexpr (CI) {
         if (threadIdx.x == 0) {
 #pragma unroll
             for (uint32_t k = 0; k < MAX_CLASS_ITEMS; k++) item_off[k] = a.mc.item_off[k];
         }
     }
+    if constexpr (CI == 2) {
+        // item k's class is the k-th residue coprime to Q
+        wc.ms = (uint32_t)(pl.M_start % a.mc.Q);
+        const uint32_t k = threadIdx.x;
+        uint32_t r = k < a.mc.items ? a.mc.item_off[k] + wc.ms : ~0u;
+        if (k < a.mc.items && r >= a.mc.Q) r -= a.mc.Q;
+        if (k < a.mc.items) rank[r] = (uint8_t)k;
+        wc.rank0 = (uint32_t)__syncthreads_count(r < wc.ms);
+    }
     if constexpr (BKT)
         for (uint32_t b = threadIdx.x; b < pl.n_bands; b += LARGE_THREADS)
             bkt_s[b] = pl.bkt_cnt[(uint64_t)b * pl.n_regions + blockIdx.x];
-    if constexpr (CI || BKT) __syncthreads();
-    walk_warp<UT, ST, MT, NC, CI, false, BKT, PRE>(a, queue[threadIdx.x >> 5], item_off,
-                                              (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) >> 5,
-                                              ((uint64_t)gridDim.x * blockDim.x) >> 5, bkt_s);
+    if constexpr (SM)
+        for (uint32_t k = threadIdx.x; k < pl.S32; k += LARGE_THREADS) mask_s[k] = __ldg(&pl.col_mask[k]);
+    if constexpr (CI || BKT || SM) __syncthreads();
+    const uint32_t wib = threadIdx.x >> 5;
+    walk_warp<UT, ST, MT, NC, CI, SM, false, BKT, PRE>(a, queue[wib], hits[wib], SM ? mask_s : pl.col_mask, wc,
+                                                       (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) >> 5,
+                                                       ((uint64_t)gridDim.x * blockDim.x) >> 5, bkt_s);
     if constexpr (BKT) {
         // the region counts for the next launch (slots past the region's end were cleared directly)
         __syncthreads();
@@ -688,8 +760,7 @@ __global__ void __launch_bounds__(APPLY_THREADS) k_apply_buckets(const DevPlan p
     }
 }
 
-// resident CTAs per SM the multi-job walk is compiled for: its hit path keeps
-// the plan's fields in registers, which at three CTAs per SM would spill
+// resident CTAs per SM the multi-job walk is compiled for
 #ifndef CS_TG_JOBS_MIN_BLOCKS
 #define CS_TG_JOBS_MIN_BLOCKS 2
 #endif
@@ -698,6 +769,7 @@ __global__ void __launch_bounds__(LARGE_THREADS, CS_TG_JOBS_MIN_BLOCKS)
     k_large_tg_jobs(const LargeArgs *jobs, uint32_t n_jobs) {
     constexpr int QCAP = 32 * (NC + 1);
     __shared__ TGItem<MT> queue[TG_WARPS][QCAP];
+    __shared__ HitBuf hits[TG_WARPS];
     __shared__ LargeArgs job[TG_WARPS];
     const unsigned lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const uint64_t warp_id = (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) >> 5;
@@ -714,7 +786,8 @@ __global__ void __launch_bounds__(LARGE_THREADS, CS_TG_JOBS_MIN_BLOCKS)
         const uint64_t n = min((uint64_t)*a.count, a.cap);
         const uint64_t batches = (n * a.n_seg * (CI ? a.mc.items : 1) + 31) / 32;
         const uint64_t first = (warp_id + n_warps - dealt % n_warps) % n_warps;
-        walk_warp<UT, ST, MT, NC, CI, true>(a, queue[wib], a.mc.item_off, first, n_warps);
+        const WalkClasses wc{a.mc.item_off, nullptr, 0, 0, 0, 0};
+        walk_warp<UT, ST, MT, NC, CI, false, true>(a, queue[wib], hits[wib], a.pl.col_mask, wc, first, n_warps);
         dealt += batches;
         __syncwarp();
     }
@@ -745,7 +818,7 @@ bool prep_eligible(const DevPlan &pl, int mode, uint32_t n_seg, MClasses mc) {
 cudaError_t launch_tg_prep(const DevPlan &pl, bool narrow, const void *p, const void *r, const void *v,
                            const unsigned long long *count, uint64_t cap, uint64_t p_lo, uint64_t p_hi,
                            MClasses mc, uint4 *desc0, uint2 *desc1, cudaStream_t stream) {
-    LargeArgs a{pl, p, r, v, count, cap, 1, p_lo, p_hi, mc, nullptr, nullptr};
+    LargeArgs a{pl, p, r, v, count, cap, 1, p_lo, p_hi, mc, nullptr, nullptr, 0, 0};
     void (*kern)(const LargeArgs, uint4 *, uint2 *) =
         narrow ? k_tg_prep<uint32_t, int32_t> : k_tg_prep<uint64_t, int64_t>;
     // one wave of resident CTAs, looked up once per width
@@ -762,6 +835,19 @@ cudaError_t launch_tg_prep(const DevPlan &pl, bool narrow, const void *p, const 
     return cudaGetLastError();
 }
 
+namespace {
+constexpr uint32_t WALK_MASK_WORDS = 4096;     // largest column mask copied to shared memory
+template <class UT, class ST, bool SM>
+void (*walk_kernel(int kind, int bkt))(const LargeArgs) {
+    if (kind == 4) return bkt ? k_large_tg<UT, ST, uint32_t, 1, 0, SM, true, true> : k_large_tg<UT, ST, uint32_t, 1, 0, SM, false, true>;
+    if constexpr (sizeof(UT) == 4)
+        if (kind == 3) return bkt ? k_large_tg<UT, ST, uint32_t, 1, 2, SM, true, false> : k_large_tg<UT, ST, uint32_t, 1, 2, SM, false, false>;
+    if (kind == 2) return bkt ? k_large_tg<UT, ST, uint32_t, 1, 1, SM, true, false> : k_large_tg<UT, ST, uint32_t, 1, 1, SM, false, false>;
+    if (kind == 1) return bkt ? k_large_tg<UT, ST, uint32_t, 2, 0, SM, true, false> : k_large_tg<UT, ST, uint32_t, 2, 0, SM, false, false>;
+    return bkt ? k_large_tg<UT, ST, uint32_t, 1, 0, SM, true, false> : k_large_tg<UT, ST, uint32_t, 1, 0, SM, false, false>;
+}
+}  // namespace
+
 cudaError_t launch_large(const DevPlan &pl, bool narrow, int mode, const void *p, const void *r,
                          const void *v, const unsigned long long *count, uint64_t cap, uint32_t n_seg,
                          int grid, cudaStream_t stream, uint64_t p_lo, uint64_t p_hi, MClasses mc,
@@ -777,52 +863,43 @@ cudaError_t launch_large(const DevPlan &pl, bool narrow, int mode, const void *p
     const bool pre = desc0 && desc1 && kind == 0 && prep_eligible(pl, mode, n_seg, mc);
     if (pre) kind = 4;
     LargeArgs a{pl, p, r, v, count, cap, n_seg ? n_seg : 1, p_lo, p_hi, mc, pre ? desc0 : nullptr,
-                pre ? desc1 : nullptr};
+                pre ? desc1 : nullptr, 0, 0};
+    if (kind == 3) magic_of(mc.Q, a.q_magic, a.q_shift);
     // bucketed hits: three-gap walk only (the paper's walk clears directly)
     const int bkt = (pl.bucket && mode != LARGE_PAPER) ? 1 : 0;
     if (!bkt) a.pl.bucket = 0;
-    const size_t dyn = bkt ? (size_t)pl.n_bands * sizeof(uint32_t) : 0;
-    void (*walk)(const LargeArgs) = nullptr;
-    if (narrow) {
-        walk = kind == 4 ? (bkt ? k_large_tg<uint32_t, int32_t, uint32_t, 1, 0, true, true>
-                                : k_large_tg<uint32_t, int32_t, uint32_t, 1, 0, false, true>)
-             : kind == 3 ? (bkt ? k_large_tg<uint32_t, int32_t, uint32_t, 1, 2, true>
-                                : k_large_tg<uint32_t, int32_t, uint32_t, 1, 2>)
-             : kind == 2 ? (bkt ? k_large_tg<uint32_t, int32_t, uint32_t, 1, 1, true>
-                                : k_large_tg<uint32_t, int32_t, uint32_t, 1, 1>)
-             : kind == 1 ? (bkt ? k_large_tg<uint32_t, int32_t, uint32_t, 2, 0, true>
-                                : k_large_tg<uint32_t, int32_t, uint32_t, 2>)
-                         : (bkt ? k_large_tg<uint32_t, int32_t, uint32_t, 1, 0, true>
-                                : k_large_tg<uint32_t, int32_t, uint32_t, 1>);
-    } else {
-        walk = kind == 4 ? (bkt ? k_large_tg<uint64_t, int64_t, uint32_t, 1, 0, true, true>
-                                : k_large_tg<uint64_t, int64_t, uint32_t, 1, 0, false, true>)
-             : kind == 2 ? (bkt ? k_large_tg<uint64_t, int64_t, uint32_t, 1, 1, true>
-                                : k_large_tg<uint64_t, int64_t, uint32_t, 1, 1>)
-             : kind == 1 ? (bkt ? k_large_tg<uint64_t, int64_t, uint32_t, 2, 0, true>
-                                : k_large_tg<uint64_t, int64_t, uint32_t, 2>)
-                         : (bkt ? k_large_tg<uint64_t, int64_t, uint32_t, 1, 0, true>
-                                : k_large_tg<uint64_t, int64_t, uint32_t, 1>);
-    }
+    // the column mask goes to shared memory up to 16 KB (SL < 65,536): its lookups, one
+    // per visited hit at random offsets, take about 3 wavefronts a warp there
+    // and about 20 in L1
+    const bool sm = pl.S32 <= WALK_MASK_WORDS;
+    const size_t dyn = ((bkt ? pl.n_bands : 0) + (sm ? pl.S32 : 0)) * sizeof(uint32_t);
+    void (*walk)(const LargeArgs) =
+        narrow ? (sm ? walk_kernel<uint32_t, int32_t, true>(kind, bkt) : walk_kernel<uint32_t, int32_t, false>(kind, bkt))
+               : (sm ? walk_kernel<uint64_t, int64_t, true>(kind, bkt) : walk_kernel<uint64_t, int64_t, false>(kind, bkt));
     // the three-gap walk's lanes are persistent: by default one wave of
     // resident CTAs (a partial last wave left SMs idle: 3% slower measured);
     // the paper's walk takes eight CTAs per SM
-    if (grid <= 0) {
-        grid = sm_count() * 8;
-        if (mode != LARGE_PAPER) {
-            // looked up once per [narrow][kind][bucketed] (the bucket counters,
-            // at most 16 KB, do not change the occupancy bound by registers)
-            static std::atomic<int> resident[2][5][2];
-            std::atomic<int> &cached = resident[narrow ? 1 : 0][kind][bkt];
-            int per_sm = cached.load(std::memory_order_relaxed);
-            if (per_sm == 0) {
-                cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, walk, LARGE_THREADS,
-                                                                              bkt ? 4 * BKT_MAX_BANDS : 0);
-                if (e != cudaSuccess || per_sm <= 0) per_sm = -1;
-                cached.store(per_sm, std::memory_order_relaxed);
-            }
-            if (per_sm > 0) grid = sm_count() * per_sm;
+    if (mode == LARGE_PAPER) {
+        if (grid <= 0) grid = sm_count() * 8;
+    } else {
+        // once per device and [narrow][kind][bucketed][mask]: the shared-memory limit
+        // raised to the most that form can take, and the CTAs resident with that
+        static std::atomic<int> resident[64][2][5][2][2];
+        int dev = 0;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e != cudaSuccess) return e;
+        if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+        std::atomic<int> &cached = resident[dev][narrow ? 1 : 0][kind][bkt][sm];
+        int per_sm = cached.load(std::memory_order_relaxed);
+        if (per_sm == 0) {
+            const int most = (int)(((bkt ? BKT_MAX_BANDS : 0) + (sm ? WALK_MASK_WORDS : 0)) * sizeof(uint32_t));
+            e = cudaFuncSetAttribute(walk, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+            if (e != cudaSuccess) return e;
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, walk, LARGE_THREADS, (size_t)most);
+            if (e != cudaSuccess || per_sm <= 0) per_sm = 1;
+            cached.store(per_sm, std::memory_order_relaxed);
         }
+        if (grid <= 0) grid = sm_count() * per_sm;
     }
     // every walking CTA owns a region per band
     if (bkt && (uint32_t)grid > pl.n_regions) grid = (int)pl.n_regions;
@@ -871,7 +948,8 @@ cudaError_t walk_jobs_create(const std::vector<WalkJob> &jobs, WalkJobs **out) {
         MClasses mc = j.mc;
         const int kind = walk_kind(mc, j.pl.SL);
         g[j.narrow ? 1 : 0][kind].push_back(
-            LargeArgs{j.pl, j.p, j.r, nullptr, j.count, j.cap, j.n_seg ? j.n_seg : 1, j.p_lo, j.p_hi, mc});
+            LargeArgs{j.pl, j.p, j.r, nullptr, j.count, j.cap, j.n_seg ? j.n_seg : 1, j.p_lo, j.p_hi, mc, nullptr, nullptr,
+                      0, 0});
         g[j.narrow ? 1 : 0][kind].back().pl.bucket = 0;      // the job walks clear directly
     }
     WalkJobs *wj = new (std::nothrow) WalkJobs();
