@@ -95,7 +95,8 @@ typedef struct {
                                 mod 210 (else 30, 6, 2: the largest that divides d) in every
                                 chunk */
     uint32_t item_hits;      /* three-gap walk: expected walked hits per work item (prime,
-                                m-segment); 0 = automatic (128) */
+                                m-segment); 0 = automatic (128, down to 16 when a chunk
+                                would not fill the GPU) */
     uint32_t class_min_hits; /* m_classes = 0: expected hits per prime (every m) from which a
                                 chunk walks only the m-classes; 0 = automatic (48) */
     uint32_t class_item_hits;/* m_classes = 0: expected hits of one class of m mod Q (Q = 210

@@ -478,8 +478,19 @@ cs_status build_plan(cs_plan_s *pl, uint32_t P, uint64_t d, uint64_t M_start, ui
         if (T < 2ull * SL || T > MAX_T)
             return fail(CS_EINVAL, "threshold must satisfy 2*SL <= T <= 2^30");
     } else {
-        uint64_t mult = pl->mode == LARGE_PAPER ? 100 : 8;
-        T = std::min<uint64_t>(std::max<uint64_t>(mult * S, 1u << 16), MAX_T);
+        // three-gap walk: 3 S (1 to 12 S measured: per sieve of search_953 7.4 to 8.5 ms,
+        // best at 1.5 to 3 S; of 333,333 multipliers of 1019#/2310 51.0 to 55.2 ms), and
+        // 65,536 at least, below which a prime costs its launches more than its marks
+        uint64_t mult = pl->mode == LARGE_PAPER ? 100 : 3;
+        T = std::max<uint64_t>(mult * S, 1u << 16);
+        if (pl->mode == LARGE_THREE_GAP && M_c > 0) {
+            // few rows: up to about 8e6 (row, prime) pairs cost the tile sieve less than
+            // the walk's chunks of primes with many hits (one per factor 2 of p, about
+            // 45 us each), so those primes move to it (K = 503#/210 to 1e7: 256 -> 194 us)
+            const double x = 8e6 / (double)M_c, pairs_T = x > 3 ? x * std::log(x) : 0.0;
+            T = std::max<uint64_t>(T, (uint64_t)std::min((double)M_inc * (double)S / 48.0 + 1.0, pairs_T));
+        }
+        T = std::min<uint64_t>(T, MAX_T);
     }
     // the large-prime walk needs p > 2*SL (at most one hit per interval)
     T = std::max<uint64_t>({T, 2ull * SL, (uint64_t)P, 2});
@@ -490,7 +501,7 @@ cs_status build_plan(cs_plan_s *pl, uint32_t P, uint64_t d, uint64_t M_start, ui
     // large primes in chunks of (T, L]: geometric (factor 2) so that the hits
     // per prime, about M_inc * S / p, vary at most 2x inside a chunk, capped at
     // chunk_numbers wide; a chunk's primes are split into n_seg m-segments of
-    // about HITS_PER_ITEM expected hits each
+    // about item_hits expected hits each
     const uint64_t chunk = pl->tune.chunk_numbers ? pl->tune.chunk_numbers : (1ull << 27);
     // m-classes per chunk (cs_classes.h): class items mod 210 or 30 for the
     // primes with the most hits, then m = 1, 5 (mod 6), then the odd m
@@ -498,16 +509,23 @@ cs_status build_plan(cs_plan_s *pl, uint32_t P, uint64_t d, uint64_t M_start, ui
     const ClassTiers tiers = class_tiers(pl->mode == LARGE_THREE_GAP && SL > 0, d, M_start, M_inc, S, pl->tune);
     pl->mcls = tiers.mcls;
     pl->mcls_light = tiers.mcls_light;
-    const double HITS_PER_ITEM = pl->tune.item_hits ? (double)pl->tune.item_hits : 128.0;
     auto classes_for = [&](uint64_t lo) -> MClasses { return tiers.for_chunk(lo); };
     // walked hits per item: a class (class items) or the item's n classes
+    const double walk_lanes = (double)sm_count() * 3 * 256;
     auto segs_for = [&](uint64_t lo) {
-        double hits = (double)M_inc * (double)S / (double)std::max<uint64_t>(lo, 1);
+        const double l = (double)std::max<uint64_t>(lo, 3);
         const MClasses mc = classes_for(lo);
-        hits *= (double)(mc.items ? 1 : mc.n) / (double)mc.Q;
+        const double scale = (double)M_inc * (double)S / (double)mc.Q;
+        const double hits = scale / l * (double)(mc.items ? 1 : mc.n);
+        // 128 hits, or as few as 16 when a chunk of several walkers per prime (lo, 2 lo]
+        // would not give every lane of the walk two items
+        double per = pl->tune.item_hits ? (double)pl->tune.item_hits : 128.0;
+        if (!pl->tune.item_hits && (mc.items || mc.n > 1))
+            per = std::max(16.0, std::min(per, scale * (double)mc.n * std::log(std::log(2 * l) / std::log(l)) /
+                                                   (2 * walk_lanes)));
         // at most 2^30 m per segment: the walk's offsets and clamped steps fit 32 bits
         const double fewest = M_inc > (1ull << 30) ? 2.0 : 1.0;
-        double seg = std::min<double>(std::max(fewest, std::ceil(hits / HITS_PER_ITEM)), (double)std::max<uint64_t>(M_inc, 1));
+        double seg = std::min<double>(std::max(fewest, std::ceil(hits / per)), (double)std::max<uint64_t>(M_inc, 1));
         return (uint32_t)std::min(seg, 65536.0);
     };
     auto add_chunk = [&](uint64_t lo, uint64_t hi) {
@@ -544,6 +562,11 @@ cs_status build_plan(cs_plan_s *pl, uint32_t P, uint64_t d, uint64_t M_start, ui
     } else {
         for (uint64_t lo = T; lo < L;) {
             uint64_t hi = std::min<uint64_t>({L, lo + std::max<uint64_t>(lo, 1), lo + chunk});
+            // one walker per prime from here on: nothing depends on the hits per prime any
+            // more, and a chunk takes its full width (three launches less each; K =
+            // 503#/210 to 1e7 takes 3 chunks instead of 7)
+            const MClasses mc = classes_for(lo);
+            if (!mc.items && mc.n == 1 && segs_for(lo) == 1) hi = std::min<uint64_t>(L, lo + chunk);
             // a chunk ends below 2^30 when the next one starts above: it keeps the
             // 32-bit kernels
             if (lo < NARROW_LIMIT - 1 && hi >= NARROW_LIMIT) hi = NARROW_LIMIT - 1;
@@ -576,11 +599,24 @@ cs_status build_plan(cs_plan_s *pl, uint32_t P, uint64_t d, uint64_t M_start, ui
         return (z1 - (z0 & ~31ull) + 31) / 32;
     };
     uint64_t full_words = W ? words_of(0, W) : 1;
-    if (!TR) {
+    const bool auto_rows = TR == 0;
+    if (auto_rows) {
+        // the most rows that leave room for two CTAs per SM (two hide each other's
+        // barriers: search_953's tile sieve 1.25 ms at 16 rows, 1.46 at 32), or for one,
+        // and then as few as it takes to give every SM two CTAs (230 rows: 92 us at 32
+        // rows a CTA, 15 at 1)
+        const uint64_t pair = (228 * 1024 / 2 - 1024 - tile_stage_bytes()) / 4;
+        const uint64_t room = 2 * full_words <= pair ? pair : budget;
         TR = 32;
-        while (TR > 1 && (uint64_t)(TR + 1) * full_words > budget) TR /= 2;
+        while (TR > 1 && (uint64_t)(TR + 1) * full_words > room) TR /= 2;
+        while (TR > 1 && (M_c + TR - 1) / TR < 2 * (uint64_t)sm_count()) TR /= 2;
     }
     uint64_t max_words_per_chunk = budget / (TR + 1);
+    // fewer rows than SMs: the columns are cut too, so that every SM has a CTA (11 rows
+    // of 9,618 columns: 450 us in one piece a row)
+    if (auto_rows && pl->layout == 0 && M_c > 0 && M_c < (uint64_t)sm_count())
+        max_words_per_chunk = std::min<uint64_t>(
+            max_words_per_chunk, std::max<uint64_t>(64, (full_words * M_c + sm_count() - 1) / sm_count()));
     if (max_words_per_chunk < 64) return fail(CS_EINVAL, "tile_rows too large for shared memory");
     if (pl->layout == 1 && (uint64_t)(TR + 1) * full_words > budget)
         return fail(CS_EINVAL, "the compact layout needs the interval's tile in one piece (smaller SL or tile_rows)");
@@ -718,7 +754,9 @@ cs_status build_plan(cs_plan_s *pl, uint32_t P, uint64_t d, uint64_t M_start, ui
     uint64_t *d_bits; uint32_t *d_cnt; unsigned long long *d_stats;
     if ((s = pl->dalloc(&d_bits, M_c * wpr))) return s;
     if ((s = pl->dalloc(&d_cnt, M_c))) return s;
-    if ((s = pl->dalloc(&d_stats, ST_COUNT))) return s;
+    // the statistics and, behind them, the prime counts (one reset per sieve)
+    if ((s = pl->dalloc(&d_stats, ST_COUNT + 1 + pl->chunks.size()))) return s;
+    pl->d_counts = d_stats + ST_COUNT;
     dp.bits = d_bits; dp.counts = d_cnt; dp.stats = d_stats;
     if (dp.bucket) {
         const uint64_t before = pl->dev_bytes;
@@ -742,7 +780,6 @@ cs_status build_plan(cs_plan_s *pl, uint32_t P, uint64_t d, uint64_t M_start, ui
     if ((s = pl->flush_uploads())) return s;
 
     if ((s = pl->dalloc(&pl->d_small, pl->small_cap))) return s;
-    if ((s = pl->dalloc(&pl->d_counts, 1 + pl->chunks.size()))) return s;
     if (!pl->chunks.empty() && !pl->cache) {
         size_t el = pl->narrow ? 4 : 8;
         uint8_t *a, *b, *c;
@@ -858,8 +895,7 @@ cs_status plan_sieve_head(cs_plan_t pl, cudaStream_t st) {
     const DevPlan &dp = pl->dp;
     Prof prof{pl, st, pl->tune.profile != 0};
     for (int k = 0; k < KC_N; k++) pl->prof_used[k] = 0;
-    CS_CUDA(cudaMemsetAsync(dp.stats, 0, ST_COUNT * sizeof(unsigned long long), st));
-    CS_CUDA(cudaMemsetAsync(pl->d_counts, 0, (1 + pl->chunks.size()) * sizeof(unsigned long long), st));
+    CS_CUDA(cudaMemsetAsync(dp.stats, 0, (ST_COUNT + 1 + pl->chunks.size()) * sizeof(unsigned long long), st));
     if (dp.bucket)
         CS_CUDA(cudaMemsetAsync(dp.bkt_cnt, 0, ((size_t)dp.n_bands * dp.n_regions + 1) * sizeof(uint32_t), st));
     cs_status s;
