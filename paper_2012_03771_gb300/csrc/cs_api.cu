@@ -302,6 +302,11 @@ cs_status check_params(uint32_t P, uint64_t d, uint64_t M_start, uint64_t M_inc,
     return CS_OK;
 }
 
+// chunk c tries every m (automatic choice only: an explicit walk_prep keeps the walk)
+bool plan_few(const cs_plan_s *pl, size_t c) {
+    return !pl->cache && !pl->tune.walk_prep && few_eligible(pl->dp, pl->mode, pl->chunk_seg[c], pl->chunk_mc[c]);
+}
+
 // tuning fields left at 0 may be set from the environment
 void env_tuning(cs_tuning &t) {
     auto get = [](const char *n) -> uint64_t {
@@ -789,7 +794,8 @@ cs_status build_plan(cs_plan_s *pl, uint32_t P, uint64_t d, uint64_t M_start, ui
         pl->d_lp = a; pl->d_lr = b; pl->d_lv = c;
         bool any_prep = false;
         for (size_t k = 0; k < pl->chunks.size(); k++)
-            any_prep = any_prep || prep_eligible(pl->dp, pl->mode, pl->chunk_seg[k], pl->chunk_mc[k]);
+            any_prep = any_prep || (prep_eligible(pl->dp, pl->mode, pl->chunk_seg[k], pl->chunk_mc[k]) &&
+                                    !plan_few(pl, k));
         if (any_prep && pl->tune.walk_prep != 1) {
             if ((s = pl->dalloc(&pl->d_desc0, pl->large_cap))) return s;
             if ((s = pl->dalloc(&pl->d_desc1, pl->large_cap))) return s;
@@ -999,6 +1005,13 @@ cs_status cs_sieve(cs_plan_t pl, void *stream) {
                                  pl->d_base, pl->n_base, pl->d_lp, pl->d_lr, pl->d_lv,
                                  pl->large_cap, cnt, st));
         if ((s = prof.end())) return s;
+        if (plan_few(pl, c)) {
+            if ((s = prof.begin(KC_LARGE))) return s;
+            CS_CUDA(launch_few(dp, narrow, pl->d_lp, pl->d_lr, pl->d_lv, cnt, pl->large_cap, pl->chunk_mc[c], st));
+            if ((s = prof.end())) return s;
+            if ((s = apply(c))) return s;
+            continue;
+        }
         const bool pre = pl->d_desc0 && prep_eligible(dp, pl->mode, pl->chunk_seg[c], pl->chunk_mc[c]);
         if (pre) {
             if ((s = prof.begin(KC_PREP))) return s;

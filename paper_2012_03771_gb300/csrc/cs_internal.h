@@ -184,6 +184,13 @@ bool prep_eligible(const DevPlan &pl, int mode, uint32_t n_seg, MClasses mc);
 cudaError_t launch_tg_prep(const DevPlan &pl, bool narrow, const void *p, const void *r, const void *v,
                            const unsigned long long *count, uint64_t cap, uint64_t p_lo, uint64_t p_hi,
                            MClasses mc, uint4 *desc0, uint2 *desc1, cudaStream_t stream);
+// The walk of one-walker chunks over few m (up to FEW_M: one addition per m costs
+// less than the preparation of a walker, about 540 instructions, up to some 200 odd
+// m): every m of the class tried, no preparation, hits cleared directly.
+constexpr uint32_t FEW_M = 256;
+bool few_eligible(const DevPlan &pl, int mode, uint32_t n_seg, MClasses mc);
+cudaError_t launch_few(const DevPlan &pl, bool narrow, const void *p, const void *r, const void *v,
+                       const unsigned long long *count, uint64_t cap, MClasses mc, cudaStream_t stream);
 cudaError_t launch_final(const DevPlan &pl, cudaStream_t stream);
 // Clears the bucketed hits of the walk launches since the last application,
 // band after band, and empties the regions.

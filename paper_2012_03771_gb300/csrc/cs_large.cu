@@ -24,6 +24,7 @@
 
 #include "cs_arith.cuh"
 #include "cs_internal.h"
+#include "cs_residue.cuh"
 #include "cs_walker.cuh"
 
 namespace cs {
@@ -48,11 +49,9 @@ struct LargeArgs {
 };
 
 // v0 = (r * M_start + SL) mod p, for primes from a shared residue cache
-__device__ __forceinline__ uint32_t start_v(uint32_t r, uint64_t M_start, uint32_t SL, uint32_t p) {
-    return (uint32_t)(((uint64_t)r * (M_start % p) + SL) % p);
-}
-__device__ __forceinline__ uint64_t start_v(uint64_t r, uint64_t M_start, uint32_t SL, uint64_t p) {
-    return (uint64_t)(((unsigned __int128)r * (M_start % p) + SL) % p);
+template <class UT>
+__device__ __forceinline__ UT start_v(UT r, uint64_t M_start, uint32_t SL, UT p) {
+    return (UT)near_affine(r, M_start, SL, p);
 }
 
 // (r * m + v) mod p for m < 2^31
@@ -706,6 +705,66 @@ __global__ void __launch_bounds__(PREP_THREADS) k_tg_prep(const LargeArgs a, uin
     }
 }
 
+// The walk of a chunk of one-walker primes over few m (M_inc <= FEW_M): no steps and
+// no first hit, every walked m is tried.  v / p as a 32-bit fraction of a turn advances
+// by a constant per step and wraps by itself, so a step is an addition and a minimum; m
+// whose fraction, with a margin for the roundings, is at most 2SL / p are then tried
+// exactly.  Bound: instruction issue, about 120 per prime at 22 odd m against 600 of the
+// preparation and the walk's descriptors: 11 rows of 1511#/210 to 1e10, preparation
+// and walk 13.0 ms, this kernel 6.0.
+constexpr int FEW_THREADS = 256;
+constexpr int FEW_PASS = 8;
+template <class UT>
+__global__ void __launch_bounds__(FEW_THREADS) k_few_m(const LargeArgs a) {
+    const DevPlan &pl = a.pl;
+    const UT *Pp = reinterpret_cast<const UT *>(a.p);
+    const UT *Rp = reinterpret_cast<const UT *>(a.r);
+    const UT *Vp = reinterpret_cast<const UT *>(a.v);
+    const uint64_t n = min((uint64_t)*a.count, a.cap);
+    const uint32_t Q = a.mc.Q, off0 = a.mc.off[0], w = 2 * pl.SL;
+    const uint32_t n_step = pl.M_inc > off0 ? ((uint32_t)pl.M_inc - off0 + Q - 1) / Q : 0;
+    // the fractions start within 2 and step within 2
+    const uint32_t margin = 2 * n_step + 4;
+    const uint64_t stride = (uint64_t)gridDim.x * FEW_THREADS;
+    Counters c;
+    for (uint64_t i = blockIdx.x * (uint64_t)FEW_THREADS + threadIdx.x; i < n; i += stride) {
+        const UT p = Pp[i], r = Rp[i], v0 = Vp[i];
+        const UT v = off0 ? add_times(v0, r, 1, p) : v0;           // off0 < Q <= 2
+        const UT rq = Q > 1 ? add_times(r, r, 1, p) : r;
+        const float rp = walker_rcp(p);
+        uint32_t u = near_frac32(v, p, rp) + margin;
+        const uint32_t du = near_frac32(rq, p, rp);
+        const float limit = (float)w * rp * 4294967296.0f * 1.000001f + (float)(2 * margin + 2);
+        const uint32_t top = limit < 4294967040.0f ? (uint32_t)limit : ~0u;
+        for (uint32_t j0 = 0; j0 < n_step; j0 += FEW_PASS) {
+            const uint32_t start = u;
+            uint32_t low = u;
+#pragma unroll
+            for (int j = 1; j < FEW_PASS; j++) {
+                u += du;
+                low = min(low, u);
+            }
+            u += du;
+            if (low > top) continue;
+            uint32_t t = start;
+            for (uint32_t j = j0; j < min(j0 + FEW_PASS, n_step); j++, t += du) {
+                if (t > top) continue;
+                const uint64_t vm = ((uint64_t)v + (uint64_t)rq * j) % p;      // j < 2^8
+                if (vm > w) continue;
+                c.hits++;
+                const uint32_t moff = off0 + Q * j, z = w - (uint32_t)vm;
+                if (bit_of(__ldg(&pl.col_mask[z >> 5]), z))
+                    take_hit<UT, false, false>(pl, moff, z, __ldg(&pl.row_tab[moff >> 5]), Pp, (uint32_t)i, c.F, nullptr);
+            }
+        }
+    }
+    const unsigned long long F = warp_sum(c.F), hits = warp_sum(c.hits);
+    if ((threadIdx.x & 31) == 0) {
+        if (F) atomicAdd(pl.stats + ST_F_LARGE, F);
+        if (hits) atomicAdd(pl.stats + ST_HITS_ALL, hits);
+    }
+}
+
 // Clears the bucketed records: each CTA takes whole regions one at a time from
 // a shared counter (bkt_cnt[n_bands * n_regions]) in band-major order, so that
 // the regions in work at one time belong to one or two consecutive bands,
@@ -813,6 +872,21 @@ __global__ void k_modsolve(const uint64_t *p, const uint64_t *K, const uint64_t 
 bool prep_eligible(const DevPlan &pl, int mode, uint32_t n_seg, MClasses mc) {
     return mode != LARGE_PAPER && pl.SL > 0 && (n_seg <= 1) && !mc.items && mc.n == 1 && mc.Q <= 2 &&
            mc.off[0] < mc.Q;
+}
+
+bool few_eligible(const DevPlan &pl, int mode, uint32_t n_seg, MClasses mc) {
+    return prep_eligible(pl, mode, n_seg, mc) && pl.M_inc <= FEW_M;
+}
+
+cudaError_t launch_few(const DevPlan &pl, bool narrow, const void *p, const void *r, const void *v,
+                       const unsigned long long *count, uint64_t cap, MClasses mc, cudaStream_t stream) {
+    LargeArgs a{pl, p, r, v, count, cap, 1, 0, ~0ull, mc, nullptr, nullptr, 0, 0};
+    a.pl.bucket = 0;                                       // clears directly
+    if (narrow)
+        k_few_m<uint32_t><<<sm_count() * 8, FEW_THREADS, 0, stream>>>(a);
+    else
+        k_few_m<uint64_t><<<sm_count() * 8, FEW_THREADS, 0, stream>>>(a);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_tg_prep(const DevPlan &pl, bool narrow, const void *p, const void *r, const void *v,

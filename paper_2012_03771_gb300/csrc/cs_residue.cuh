@@ -127,4 +127,44 @@ CS_HD uint64_t res_affine(uint64_t r, uint64_t M, uint32_t s, const ResMod &q) {
     return x >= (int64_t)q.p ? (uint64_t)x - q.p : (uint64_t)x;
 }
 
+// x - k p for the integer k nearest to the float quotient, any p < 2^40, |x / p| <
+// 2.5 2^20, |x| < 2^62 (rp within 2^-22 of 1 / p): the quotient is off by less than
+// 1.4, so the result is within 1.5 p.
+CS_HD int64_t near_rem(int64_t x, uint64_t p, float rp) {
+#if defined(__CUDA_ARCH__)
+    const float f = __fmaf_rn((float)(int32_t)(x >> 32), 4294967296.0f, (float)(uint32_t)x);
+    const int32_t k = __float2int_rn(f * rp);
+#else
+    const float f = (float)(int32_t)(x >> 32) * 4294967296.0f + (float)(uint32_t)x;
+    const int32_t k = (int32_t)lrintf(f * rp);
+#endif
+    return x - (int64_t)k * (int64_t)p;
+}
+// (r M + s) mod p for r < p < 2^40, M < 2^40, s <= p, as res_affine
+CS_HD uint64_t near_affine(uint64_t r, uint64_t M, uint32_t s, uint64_t p) {
+    const float rp = rcp_rn(u64_to_f(p));
+    int64_t x = 0;
+    if (M >> 20) x = near_rem((int64_t)(r * (M >> 20)), p, rp);
+    if (x < 0) x += (int64_t)p;              // so that the halves of the next float do not cancel
+    x = near_rem((int64_t)(((uint64_t)x << 20) + r * (M & 0xfffffu)), p, rp) + (int64_t)s;
+    if (x < 0) x += (int64_t)p;
+    if (x < 0) x += (int64_t)p;
+    if (x >= (int64_t)p) x -= (int64_t)p;
+    if (x >= (int64_t)p) x -= (int64_t)p;
+    return (uint64_t)x;
+}
+
+// x 2^32 / p within 2, modulo 2^32, for x < p < 2^40: 16 bits of the
+// quotient at a time
+CS_HD uint32_t near_frac32(uint64_t x, uint64_t p, float rp) {
+    int32_t k1 = (int32_t)(u64_to_f(x) * 65536.0f * rp);
+    int64_t r1 = (int64_t)((x << 16) - (uint64_t)k1 * p);
+    if (r1 < 0) {
+        r1 += (int64_t)p;
+        k1--;
+    }
+    const int32_t k2 = (int32_t)(u64_to_f((uint64_t)r1) * 65536.0f * rp);
+    return ((uint32_t)k1 << 16) + (uint32_t)k2;
+}
+
 }  // namespace cs

@@ -1,7 +1,8 @@
 // Host build of the 64-bit primes' residues (cs_residue.cuh) and K's limbs
 // (cs_words.h): reads "p M s n q_1 .. q_n" lines (K = product of the q), prints
-// "r v chain": r = K mod p, v = (r M + s) mod p, and 1 when the chain of whole-sum
-// products took p (else the stepwise one).
+// "r v chain v' f": r = K mod p, v = (r M + s) mod p, 1 when the chain of whole-sum
+// products took p (else the stepwise one), v by near_affine, and r 2^32 / p by
+// near_frac32.
 #include <cstdint>
 #include <cstdio>
 #include <vector>
@@ -17,7 +18,8 @@ static void one(uint64_t p, uint64_t M, uint32_t s, const std::vector<uint32_t> 
     for (uint32_t i = 0; i < n; i++)
         t = chain ? cs::res_limb<P32>(t, i + 1 < n ? k[i + 1] : 0, q) : cs::res_step<P32>(t + k[i], q);
     const uint64_t r = cs::res_finish<P32>(t, n, q);
-    printf("%llu %llu %d\n", (unsigned long long)r, (unsigned long long)cs::res_affine<P32>(r, M, s, q), chain);
+    printf("%llu %llu %d %llu %u\n", (unsigned long long)r, (unsigned long long)cs::res_affine<P32>(r, M, s, q), chain,
+           (unsigned long long)cs::near_affine(r, M, s, p), cs::near_frac32(r, p, cs::rcp_rn(cs::u64_to_f(p))));
 }
 
 int main() {

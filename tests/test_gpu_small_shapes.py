@@ -31,3 +31,23 @@ def test_small_searches_match_oracle(P, d, M_inc, SL, L):
             assert np.array_equal(plan.bitset(), bits_ref), kw
             assert F == int(F_ref.sum()) and h == O.bitset_hash(bits_ref)
             assert np.array_equal(counts, O.row_counts(bits_ref))
+
+
+@pytest.mark.parametrize("M_inc", [1, 2, 9, 16, 17, 255, 256, 257])
+@pytest.mark.parametrize("P, d, L, threshold", [(101, 6, 300_000, 700), (101, 15, 300_000, 700), (503, 210, 1_100_000_000, 0)])
+def test_few_m_equal_prepared_walkers(P, d, L, threshold, M_inc):
+    """Chunks over few m, where every m is tried, against the walk's prepared
+    walkers: odd m and every m, 32-bit primes and some above 2^30, at the edges of
+    a pass and of the range that takes this form."""
+    for SL in (300, 9000):
+        args = (P, d, 10**6 + 3, M_inc, SL, L)
+        out = []
+        for prep in (0, 2):
+            with cs.Plan(*args, threshold=max(threshold, 2 * SL), walk_prep=prep) as plan:
+                plan.sieve(torch.cuda.current_stream()).sync()
+                assert prep or M_inc > 256 or plan.info.prep_chunks == 0
+                out.append((plan.bitset(), plan.counts(), plan.stats()))
+        assert np.array_equal(out[0][0], out[1][0])
+        assert out[0][1][1:] == out[1][1][1:]
+        for k in ("F_small", "F_large", "hits_all"):
+            assert out[0][2][k] == out[1][2][k]

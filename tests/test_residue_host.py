@@ -30,7 +30,8 @@ def test_residues_equal_exact_integers(tmp_path):
     out = subprocess.run([exe], input=text, capture_output=True, text=True, check=True).stdout.split("\n")
     ways = set()
     for (p, M, s, K), line in zip(cases, out):
-        r, v, chain = (int(x) for x in line.split())
+        r, v, chain, v2, f = (int(x) for x in line.split())
+        assert v2 == v and (f - (r << 32) // p + 2) % 2**32 <= 4, (p, M, s, len(K))
         assert (r, v) == (math.prod(K) % p, (math.prod(K) * M + s) % p), (p, M, s, len(K))
         ways.add(chain)
     assert ways == {0, 1}
