@@ -5,7 +5,7 @@
 // makes the sum divisible.  After n limbs s = K 2^(-32 n) (mod p): a limb costs three multiplies (two for p < 2^32), against the two full 64-bit
 // products per 64-bit word of a Montgomery product over K's factors.  2^(32 n)
 // is put back by one product with 2^(32 n + 64) mod p, which takes a power of two
-// near n + 64 from float quotients and five squarings.
+// near 2 n + 64 from float quotients and four squarings.
 #pragma once
 #include <stdint.h>
 
@@ -58,12 +58,17 @@ CS_HD uint64_t res_limb(uint64_t t, uint32_t next, const ResMod &q) {
     return P32 ? (uint64_t)h + next : (uint64_t)m * q.p1 + h + next;
 }
 
-// a b 2^-64 mod p, below p + 2^20, for a, b < 2^41 (P32: a, b < 2^33).  In two
-// words: (a0 b + m p) / 2^32 <= 2^41 + p, plus a1 b < 2^50 before the second step.
+// a b 2^-64 mod p, below p + 2^20, for a, b < 2^41.  In two words: (a0 b + m p) /
+// 2^32 <= 2^41 + p, plus a1 b < 2^50 before the second step.  P32: at most p + 1, for
+// a, b <= p + 1 (below 2^32): (a b + m p) / 2^32 < 2^33, and (2^33 + m p) / 2^32 < p + 2.
 template <bool P32>
 CS_HD uint64_t res_mul(uint64_t a, uint64_t b, const ResMod &q) {
     const uint32_t a0 = (uint32_t)a, a1 = (uint32_t)(a >> 32), b0 = (uint32_t)b, b1 = (uint32_t)(b >> 32);
     const uint64_t x = (uint64_t)a0 * b0;
+    if (P32) {
+        const uint64_t t = (x >> 32) + (((uint64_t)((uint32_t)x * q.ninv) * q.p0 + (uint32_t)x) >> 32);
+        return ((uint64_t)((uint32_t)t * q.ninv) * q.p0 + t) >> 32;
+    }
     const uint32_t m = (uint32_t)x * q.ninv;
     const uint64_t u = (uint64_t)m * q.p0 + (uint32_t)x;
     uint64_t t = (x >> 32) + (u >> 32) + (uint64_t)a0 * b1 + (uint64_t)a1 * b0 + ((uint64_t)(a1 * b1) << 32);
@@ -86,24 +91,25 @@ CS_HD int64_t res_near(int64_t x, const ResMod &q) {
     return x - (int64_t)k * (int64_t)q.p;
 }
 
-// 2^e mod p up to a multiple of p, in [0, 1.4 p), for e >= 39: 2^20 .. 2^39, then
-// 2^20 at a time
+// 2^e mod p up to a multiple of p, in [0, 1.4 p) (P32: below p), for e >= 39: 2^20 ..
+// 2^39, then 2^20 at a time
 template <bool P32>
 CS_HD uint64_t res_pow2(uint32_t e, const ResMod &q) {
     uint32_t done = 20 + e % 20;
     int64_t x = res_near<P32>((int64_t)1 << done, q);
     for (; done < e; done += 20) x = res_near<P32>((int64_t)((uint64_t)x << 20), q);
-    return (uint64_t)(x < 0 ? x + (int64_t)q.p : x);
+    if (x < 0) x += (int64_t)q.p;
+    return (uint64_t)(P32 && x >= (int64_t)q.p ? x - (int64_t)q.p : x);
 }
 
 // 2^(32 n + 64) mod p up to a multiple of p (below p + 2^20): with the product's
-// 2^-64, squaring takes 2^(64 + d) to 2^(64 + 2 d), so five squarings take
-// 2^(64 + n) there.
+// 2^-64, squaring takes 2^(64 + d) to 2^(64 + 2 d), so four squarings take
+// 2^(64 + 2 n) there (a squaring costs as much as three steps of 2^20).
 template <bool P32>
 CS_HD uint64_t res_back(uint32_t n, const ResMod &q) {
-    uint64_t y = res_pow2<P32>(n + 64, q);
+    uint64_t y = res_pow2<P32>(2 * n + 64, q);
 #pragma unroll
-    for (int k = 0; k < 5; k++) y = res_mul<P32>(y, y, q);
+    for (int k = 0; k < 4; k++) y = res_mul<P32>(y, y, q);
     return y;
 }
 
