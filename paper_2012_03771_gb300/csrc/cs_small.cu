@@ -59,6 +59,13 @@ __device__ __forceinline__ void bulk_to_shared(void *dst, const void *src, uint3
                  "l"((unsigned long long)__cvta_generic_to_global(src)), "r"(bytes), "r"(smem_u32(bar))
                  : "memory");
 }
+// and of a shared word, where hit is not 0, without a branch (a third of a warp's
+// marks are stored columns: the branch around each atomic cost more than the atomic)
+__device__ __forceinline__ void clear_if(uint32_t hit, uint32_t addr, uint32_t keep) {
+    asm volatile("{\n .reg .pred q;\n setp.ne.u32 q, %0, 0;\n @q red.shared::cta.and.b32 [%1], %2;\n}" ::"r"(hit), "r"(addr),
+                 "r"(keep)
+                 : "memory");
+}
 // waits for the phase with the given parity; false after max_tries polls
 __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, uint32_t max_tries) {
     for (uint32_t t = 0; t < max_tries; t++) {
@@ -147,7 +154,7 @@ __global__ void __launch_bounds__(TILE_THREADS) k_tile(const TileArgs a) {
     //    group; the prime records come into two shared-memory buffers by bulk
     //    asynchronous copies, the next one loading while the current one is
     //    used, so that the inner loop reads them with shared-memory latency
-    unsigned long long F = 0;
+    uint32_t F = 0;                // at most the marks of a row
     {
         const uint32_t stage_off = ((TR + 1) * a.tc.max_words + 3) & ~3u;      // 16-byte aligned
         SmallPrime *stage = reinterpret_cast<SmallPrime *>(smem + stage_off);
@@ -176,6 +183,9 @@ __global__ void __launch_bounds__(TILE_THREADS) k_tile(const TileArgs a) {
         unsigned __int128 lowest = 0;
         if (pl.small_n) lowest = (unsigned __int128)(pl.M_start + moff) * pl.K64 - pl.SL;
         const uint32_t two_sl = 2 * pl.SL;
+        uint32_t *row = tile + r * nw;
+        const uint32_t row_s = smem_u32(row);
+        const int32_t zlo = (int32_t)(z0 - zb);
         bool failed = false;                       // a wait gave up: no more copies, no more waits
         uint32_t issued = n_st < 2 ? n_st : 2;     // stages whose copies were issued
         uint32_t fail_st = n_st;                   // first stage whose wait gave up
@@ -197,13 +207,22 @@ __global__ void __launch_bounds__(TILE_THREADS) k_tile(const TileArgs a) {
                 if (v > two_sl) continue;
                 int32_t z = (int32_t)(two_sl - v);
                 if ((uint32_t)z >= z1) z -= (int32_t)(((uint32_t)z - z1) / e.p + 1) * (int32_t)e.p;
-                for (; z >= (int32_t)z0; z -= (int32_t)e.p) {
-                    const uint32_t zz = (uint32_t)z - zb;
-                    const uint32_t bit = 1u << (zz & 31);
-                    if (!(mask[zz >> 5] & bit)) continue;
-                    if (pl.small_n && lowest + (unsigned)z == (unsigned __int128)e.p) continue;
-                    atomicAnd(&tile[r * nw + (zz >> 5)], ~bit);
-                    F++;
+                if (pl.small_n) {
+                    for (; z >= (int32_t)z0; z -= (int32_t)e.p) {
+                        const uint32_t zz = (uint32_t)z - zb;
+                        const uint32_t bit = 1u << (zz & 31);
+                        if (!(mask[zz >> 5] & bit)) continue;
+                        if (lowest + (unsigned)z == (unsigned __int128)e.p) continue;
+                        atomicAnd(&row[zz >> 5], ~bit);
+                        F++;
+                    }
+                    continue;
+                }
+                // marks p apart at zz = z - zb
+                for (int32_t zz = z - (int32_t)zb; zz >= zlo; zz -= (int32_t)e.p) {
+                    const uint32_t k = (uint32_t)zz >> 5, hit = bit_of(mask[k], (uint32_t)zz);
+                    F += hit;
+                    clear_if(hit, row_s + 4 * k, ~bit_at((uint32_t)zz));
                 }
             }
             // every thread is done with this buffer before it is loaded again
@@ -264,8 +283,8 @@ __global__ void __launch_bounds__(TILE_THREADS) k_tile(const TileArgs a) {
         }
     }
 
-    F = warp_sum(F);
-    if (lane == 0 && F) atomicAdd(pl.stats + ST_F_SMALL, F);
+    const unsigned long long F_all = warp_sum(F);
+    if (lane == 0 && F_all) atomicAdd(pl.stats + ST_F_SMALL, F_all);
 }
 
 }  // namespace
