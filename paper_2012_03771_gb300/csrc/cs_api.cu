@@ -304,7 +304,11 @@ cs_status check_params(uint32_t P, uint64_t d, uint64_t M_start, uint64_t M_inc,
 
 // chunk c tries every m (automatic choice only: an explicit walk_prep keeps the walk)
 bool plan_few(const cs_plan_s *pl, size_t c) {
-    return !pl->cache && !pl->tune.walk_prep && few_eligible(pl->dp, pl->mode, pl->chunk_seg[c], pl->chunk_mc[c]);
+    return !pl->cache && !pl->tune.walk_prep && few_eligible(pl->dp, pl->mode, pl->chunks[c].first, pl->chunk_seg[c], pl->chunk_mc[c]);
+}
+// chunk c's walkers are prepared ahead (once the plan is built)
+bool plan_prepares(const cs_plan_s *pl, size_t c) {
+    return pl->d_desc0 && prep_eligible(pl->dp, pl->mode, pl->chunk_seg[c], pl->chunk_mc[c]) && !plan_few(pl, c);
 }
 
 // tuning fields left at 0 may be set from the environment
@@ -571,7 +575,12 @@ cs_status build_plan(cs_plan_s *pl, uint32_t P, uint64_t d, uint64_t M_start, ui
             // more, and a chunk takes its full width (three launches less each; K =
             // 503#/210 to 1e7 takes 3 chunks instead of 7)
             const MClasses mc = classes_for(lo);
-            if (!mc.items && mc.n == 1 && segs_for(lo) == 1) hi = std::min<uint64_t>(L, lo + chunk);
+            if (!mc.items && mc.n == 1 && segs_for(lo) == 1) {
+                hi = std::min<uint64_t>(L, lo + chunk);
+                // (few m: up to the primes that take every m)
+                const uint64_t from = few_from(M_inc, S, mc);
+                if (M_inc <= FEW_M && lo < from && from < hi) hi = from;
+            }
             // a chunk ends below 2^30 when the next one starts above: it keeps the
             // 32-bit kernels
             if (lo < NARROW_LIMIT - 1 && hi >= NARROW_LIMIT) hi = NARROW_LIMIT - 1;
@@ -688,7 +697,11 @@ cs_status build_plan(cs_plan_s *pl, uint32_t P, uint64_t d, uint64_t M_start, ui
             dp.n_bands = (uint32_t)b.n_bands;
             dp.n_regions = (uint32_t)b.n_regions;
             dp.region_cap = (uint32_t)b.cap;
-            pl->apply_after = apply_groups(pl->chunks, M_c, W, b);
+            // records are the hits the wheel leaves
+            double kept = (double)W;
+            for (uint32_t q : wq)
+                if (q <= 11) kept *= 1.0 - 1.0 / (double)q;
+            pl->apply_after = apply_groups(pl->chunks, M_c, (uint64_t)std::ceil(kept), b);
             for (uint8_t f : pl->apply_after) pl->apply_launches += f;
         }
     }
@@ -1012,7 +1025,7 @@ cs_status cs_sieve(cs_plan_t pl, void *stream) {
             if ((s = apply(c))) return s;
             continue;
         }
-        const bool pre = pl->d_desc0 && prep_eligible(dp, pl->mode, pl->chunk_seg[c], pl->chunk_mc[c]);
+        const bool pre = plan_prepares(pl, c);
         if (pre) {
             if ((s = prof.begin(KC_PREP))) return s;
             CS_CUDA(launch_tg_prep(dp, narrow, pl->d_lp, pl->d_lr, pl->d_lv, cnt, pl->large_cap, 0, ~0ull,
@@ -1068,7 +1081,7 @@ cs_status cs_info(cs_plan_t pl, cs_info_t *out) {
     for (size_t c = 0; c < pl->chunks.size(); c++) {
         const auto &ch = pl->chunks[c];
         large_launches += pl->cache ? 1 : (pl->narrow || ch.second < NARROW_LIMIT) ? 2 : 3;
-        large_launches += pl->d_desc0 && prep_eligible(pl->dp, pl->mode, pl->chunk_seg[c], pl->chunk_mc[c]);
+        large_launches += plan_prepares(pl, c);
     }
     out->launches_per_sieve = (pl->small_hi > pl->P ? 1 : 0) + (pl->M_c && pl->W ? 1 : 0) +
                               (pl->M_c ? 1 : 0) + large_launches + (pl->dp.bucket ? pl->apply_launches : 0);
@@ -1089,7 +1102,7 @@ cs_status cs_info(cs_plan_t pl, cs_info_t *out) {
     out->apply_launches = pl->dp.bucket ? pl->apply_launches : 0;
     out->prep_chunks = 0;
     for (size_t c = 0; c < pl->chunks.size() && pl->d_desc0; c++)
-        out->prep_chunks += prep_eligible(pl->dp, pl->mode, pl->chunk_seg[c], pl->chunk_mc[c]);
+        out->prep_chunks += plan_prepares(pl, c);
     if (pl->layout == 1) out->W = pl->Wc_max;
     return CS_OK;
 }

@@ -552,9 +552,8 @@ __device__ __forceinline__ void walk_warp(const LargeArgs &a, TGItem<MT> *q, Hit
         uint32_t cw = SM ? col_mask[z >> 5] : __ldg(&col_mask[z >> 5]);
 #pragma unroll 1
         for (int u = 0; u < STEPS; u += TG_UNROLL) {
-            bool push[TG_UNROLL];
+            uint32_t okm = 0;                        // bit v: step v is pushed
             uint2 at[TG_UNROLL];
-            uint32_t n_push = 0;
 #pragma unroll
             for (int v = 0; v < TG_UNROLL; v++) {
                 // an idle lane stays where it is (z remains a valid offset)
@@ -565,29 +564,28 @@ __device__ __forceinline__ void walk_warp(const LargeArgs &a, TGItem<MT> *q, Hit
                 if (down) zn += da, mn += ma;
                 if (up) zn -= ub, mn += mb;
                 const uint32_t cwn = SM ? col_mask[zn >> 5] : __ldg(&col_mask[zn >> 5]);
-                const bool ok = act && bit_of(cw, z);
+                uint32_t ok = bit_of(cw, z);
+                if (!act) ok = 0;
                 c.hits += act;                       // one visited hit per step taken
-                push[v] = ok;
-                if constexpr (ROWS) {
-                    if (!pl.small_n) {
-                        // a row: counted here, and even N + x need no clear
-                        c.F += ok;
-                        push[v] = ok && ((z ^ pl.SL) & pl.wh_even) == 0;
-                    }
+                if (ROWS && !pl.small_n) {
+                    // a row: counted here, and even N + x need no clear
+                    c.F += ok;
+                    ok &= ~(z ^ pl.SL) | ~pl.wh_even;
                 }
+                okm |= ok << v;
                 at[v] = make_uint2(moff, z);
-                n_push += push[v];
                 z = zn;
                 cw = cwn;
                 moff = mn;
             }
             // the lanes' places in the buffer, from ballots of their counts' bits
+            const uint32_t n_push = __popc(okm);
             const unsigned b0 = __ballot_sync(0xffffffffu, n_push & 1), b1 = __ballot_sync(0xffffffffu, n_push & 2),
                            b2 = __ballot_sync(0xffffffffu, n_push & 4);
             uint32_t slot = n_buf + __popc(b0 & lt_mask) + 2 * __popc(b1 & lt_mask) + 4 * __popc(b2 & lt_mask);
 #pragma unroll
             for (int v = 0; v < TG_UNROLL; v++)
-                if (push[v]) {
+                if (okm >> v & 1) {
                     buf.hit[slot] = at[v];
                     if (pl.small_n) buf.idx[slot] = idx;
                     slot++;
@@ -710,7 +708,8 @@ __global__ void __launch_bounds__(PREP_THREADS) k_tg_prep(const LargeArgs a, uin
 // by a constant per step and wraps by itself, so a step is an addition and a minimum; m
 // whose fraction, with a margin for the roundings, is at most 2SL / p are then tried
 // exactly.  Bound: instruction issue, about 120 per prime at 22 odd m against 600 of the
-// preparation and the walk's descriptors: 11 rows of 1511#/210 to 1e10, preparation
+// preparation and the walk's descriptors (for primes with less than one expected hit:
+// the exact tries diverge): 11 rows of 1511#/210 to 1e10, preparation
 // and walk 13.0 ms, this kernel 6.0.
 constexpr int FEW_THREADS = 256;
 constexpr int FEW_PASS = 8;
@@ -874,8 +873,8 @@ bool prep_eligible(const DevPlan &pl, int mode, uint32_t n_seg, MClasses mc) {
            mc.off[0] < mc.Q;
 }
 
-bool few_eligible(const DevPlan &pl, int mode, uint32_t n_seg, MClasses mc) {
-    return prep_eligible(pl, mode, n_seg, mc) && pl.M_inc <= FEW_M;
+bool few_eligible(const DevPlan &pl, int mode, uint64_t lo, uint32_t n_seg, MClasses mc) {
+    return prep_eligible(pl, mode, n_seg, mc) && pl.M_inc <= FEW_M && lo >= few_from(pl.M_inc, pl.S, mc);
 }
 
 cudaError_t launch_few(const DevPlan &pl, bool narrow, const void *p, const void *r, const void *v,
