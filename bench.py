@@ -377,7 +377,7 @@ def csrc_sha() -> str:
     whether stored ncu counters still apply to the built code."""
     import hashlib
     h = hashlib.sha256()
-    for name in ("cs_large.cu", "cs_arith.cuh", "cs_internal.h", "cs_walker.cuh"):
+    for name in ("cs_large.cu", "cs_arith.cuh", "cs_basis.cuh", "cs_internal.h", "cs_residue.cuh", "cs_walker.cuh"):
         f = os.path.join(ROOT, "paper_2012_03771_gb300", "csrc", name)
         h.update(name.encode())
         with open(f, "rb") as fh:
@@ -397,17 +397,16 @@ def csrc_sha() -> str:
 # constants for the walk sources whose digest is recorded (csrc_sha) and the
 # same threshold, tile height and chunking; otherwise they are not used.
 WALK_COUNTERS = {
-    # one GB300, walk sources with hit buckets, class-item rows from the steps and
-    # prepared walkers for the one-walker chunks (large_1019 buckets its hits,
-    # search_953 clears directly); prep_*: the walker-preparation kernel of the
-    # same run; large_1019's DRAM bytes were not captured at full size (several
-    # passes on a 13 GB working set)
-    "large_1019": {"csrc_sha": "c62acc85a540bf78", "threshold": 100002, "tile_rows": 8, "launches": 756,
-                   "thread_inst": 8482416284364.0, "dram_bytes": None,
-                   "prep_launches": 668, "prep_thread_inst": 3688559218341.0},
-    "search_953": {"csrc_sha": "c62acc85a540bf78", "threshold": 120003, "tile_rows": 16, "launches": 17,
-                   "thread_inst": 59499229837.0, "dram_bytes": 1798157568.0,
-                   "prep_launches": 7, "prep_thread_inst": 25639266207.0},
+    # one GB300, walk sources whose lanes step together and buffer their stored
+    # visits (large_1019 buckets its clears, search_953 clears directly); prep_*: the
+    # walker-preparation kernel of the same run; large_1019's DRAM bytes were not
+    # captured at full size (several passes on a 13 GB working set)
+    "large_1019": {"csrc_sha": "58bfec8b3616bf72", "threshold": 100002, "tile_rows": 8, "launches": 756,
+                   "thread_inst": 9043307908990.0, "dram_bytes": None,
+                   "prep_launches": 668, "prep_thread_inst": 1932755864669.0},
+    "search_953": {"csrc_sha": "58bfec8b3616bf72", "threshold": 120003, "tile_rows": 16, "launches": 17,
+                   "thread_inst": 66209562636.0, "dram_bytes": 1742188544.0,
+                   "prep_launches": 7, "prep_thread_inst": 15563575454.0},
 }
 
 

@@ -743,8 +743,10 @@ cs_status build_plan(cs_plan_s *pl, uint32_t P, uint64_t d, uint64_t M_start, ui
             else if (q <= 11) W *= q;
         }
         std::vector<uint32_t> keep((W + 31) / 32, 0);
-        for (uint64_t k = 0; k < W; k++)
-            if (std::gcd(k, W) == 1) keep[k >> 5] |= 1u << (k & 31);
+        for (auto &w : keep) w = ~0u;
+        for (uint32_t q : wq)
+            if (q != 2 && q <= 11)
+                for (uint64_t k = 0; k < W; k += q) keep[k >> 5] &= ~(1u << (k & 31));
         if (W > 1) {
             uint64_t km = 1;
             for (uint32_t q : qK) km = km * q % W;

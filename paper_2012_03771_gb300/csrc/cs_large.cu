@@ -16,8 +16,9 @@
 //                    "Continued fractions and lattice sieving", SHARCS 2005), so
 //                    after the first hit every further hit costs O(1).
 //
-// Each hit on a coprime m and a stored x clears one bit of the device bitset
-// with a 32-bit atomic AND and counts one enumerated factor.
+// Each hit on a coprime m and a stored x counts one enumerated factor and, unless
+// the wheel of d's primes has cleared its cell already, clears one bit of the device
+// bitset (a 32-bit atomic AND, or a record for the apply kernel).
 #include <atomic>
 #include <new>
 #include <vector>
@@ -266,14 +267,14 @@ struct WalkClasses {
 // and the two walkers mod 6): their m-segments hold nearly the same number of
 // hits (about the walked hits per item, 128), so the lanes of a warp finish
 // their walkers at nearly the same time and waiting for them costs little,
-// while each queue check costs its ballots and branches.  large_1019 walk: 720
-// ms at 8 steps, 689 at 16, 656 at 48, 625 at 128, 617-618 at 256 and more;
-// search_953 (fewer hits per item): 4.14, 4.08, 4.13, 4.10, 4.20-4.48 ms.
+// while each queue check costs its ballots and branches.  large_1019 walk: 475
+// ms at 64 steps, 454 at 128; search_953 3.60 and 3.59 ms.
 #ifndef CS_TG_STEPS
 #define CS_TG_STEPS 128
 #endif
-// one-walker items (odd m or every m; the light chunks, a few hits per walker):
-// four steps measured best of 2, 3, 4, 6, 8
+// one-walker items (odd m or every m; the light chunks, a few hits per walker): one
+// pass (two passes: large_1019 walk 459 against 462 ms, 333,333 multipliers of
+// 1019#/2310 18.9 against 18.4 ms)
 #ifndef CS_TG_STEPS_ALL_M
 #define CS_TG_STEPS_ALL_M 4
 #endif
@@ -292,13 +293,12 @@ __device__ __forceinline__ uint64_t mul_add_mod(uint64_t v, uint64_t r, uint32_t
     return advance(v, r, k, p);
 }
 
-// resident CTAs per SM the 32-bit walk is compiled for: three (85 registers)
-// measured 7% faster than four (64 registers, with spills) on a GB300
+// resident CTAs per SM the 32-bit walk is compiled for: three (80 registers, 454 ms
+// of walk on large_1019) against four (64 registers, 472 ms)
 #ifndef CS_TG_MIN_BLOCKS
 #define CS_TG_MIN_BLOCKS 3
 #endif
-// the same for the 64-bit walk (primes above 2^30): three CTAs (80 registers,
-// a few spills) measured 19% faster than one (136-154 registers) on L = 1e11
+// the same for the 64-bit walk (primes above 2^30; with four 490 ms, both widths)
 #ifndef CS_TG_MIN_BLOCKS_WIDE
 #define CS_TG_MIN_BLOCKS_WIDE 3
 #endif
@@ -663,10 +663,12 @@ __global__ void __launch_bounds__(LARGE_THREADS, sizeof(UT) == 4 ? CS_TG_MIN_BLO
 // segment per prime): per prime, the class's first v, the two steps from one
 // Euclid run and the first hit, exactly as the walk prepares an item, written
 // as a descriptor that the walk reads instead.  The Euclid runs are serial
-// chains of float-estimate divisions (one per step, about a dozen steps per
-// prime); the walk kernel, with its queue and hit path, holds 80 registers and
-// keeps 24 warps per SM, too few to hide them, while this kernel keeps one
-// prime per thread and many more warps.  Solver statistics and errors are
+// chains (a reciprocal, a multiply-add and two integer multiply-adds per step, 7 to
+// 9 steps per prime); the walk kernel, with its queue and buffer, holds 80 registers
+// and keeps 24 warps per SM, too few to hide them, while this kernel keeps one
+// prime per thread.  Bound: instruction issue (70% of issue slots, 568 warp
+// instructions per 32 primes).  large_1019, 3.66e9 primes: 384 ms with floor
+// quotients and 64-bit first hits, 92 ms now.  Solver statistics and errors are
 // counted here.
 constexpr int PREP_THREADS = 256;
 template <class UT, class ST>
@@ -682,12 +684,25 @@ __global__ void __launch_bounds__(PREP_THREADS) k_tg_prep(const LargeArgs a, uin
     const uint32_t max_iter = 4 * 8 * sizeof(UT) + 8;
     unsigned long long solves = 0, levels = 0, err = 0;
     const uint64_t stride = (uint64_t)gridDim.x * PREP_THREADS;
-    for (uint64_t i = blockIdx.x * (uint64_t)PREP_THREADS + threadIdx.x; i < n; i += stride) {
-        const UT pp = Pp[i], r = Rp[i];
+    // the next prime's words load while this one's chain runs (their latency was a
+    // third of the stalls: 22 -> 20 ps per prime on 32- and 64-bit chunks alike)
+    UT p_next = 0, r_next = 0, v_next = 0;
+    auto load = [&](uint64_t i) {
+        if (i < n) {
+            p_next = Pp[i];
+            r_next = Rp[i];
+            if (Vp) v_next = Vp[i];
+        }
+    };
+    const uint64_t i_first = blockIdx.x * (uint64_t)PREP_THREADS + threadIdx.x;
+    load(i_first);
+    for (uint64_t i = i_first; i < n; i += stride) {
+        const UT pp = p_next, r = r_next, v_in = v_next;
+        load(i + stride);
         uint4 d0 = make_uint4(NO_WALKER, 0, 0, 0);
         uint2 d1 = make_uint2(0, 0);
         if ((uint64_t)pp > a.p_lo && (uint64_t)pp <= a.p_hi) {
-            const UT vv = Vp ? Vp[i] : start_v(r, pl.M_start, pl.SL, pp);
+            const UT vv = Vp ? v_in : start_v(r, pl.M_start, pl.SL, pp);
             prep_walker<UT>(pp, r, vv, w, M, Q, off0, max_iter, solves, levels, err, d0, d1);
         }
         desc0[i] = d0;
@@ -726,8 +741,19 @@ __global__ void __launch_bounds__(FEW_THREADS) k_few_m(const LargeArgs a) {
     const uint32_t margin = 2 * n_step + 4;
     const uint64_t stride = (uint64_t)gridDim.x * FEW_THREADS;
     Counters c;
-    for (uint64_t i = blockIdx.x * (uint64_t)FEW_THREADS + threadIdx.x; i < n; i += stride) {
-        const UT p = Pp[i], r = Rp[i], v0 = Vp[i];
+    UT p_next = 0, r_next = 0, v_next = 0;
+    auto load = [&](uint64_t i) {
+        if (i < n) {
+            p_next = Pp[i];
+            r_next = Rp[i];
+            v_next = Vp[i];
+        }
+    };
+    const uint64_t i_first = blockIdx.x * (uint64_t)FEW_THREADS + threadIdx.x;
+    load(i_first);
+    for (uint64_t i = i_first; i < n; i += stride) {
+        const UT p = p_next, r = r_next, v0 = v_next;
+        load(i + stride);                                          // in flight meanwhile
         const UT v = off0 ? add_times(v0, r, 1, p) : v0;           // off0 < Q <= 2
         const UT rq = Q > 1 ? add_times(r, r, 1, p) : r;
         const float rp = walker_rcp(p);
