@@ -161,15 +161,16 @@ typedef struct {
     uint64_t F_small;
     uint64_t F_large;
     uint64_t solves;           /* G solves of Eq. modeq in the large-prime walk */
-    uint64_t levels;           /* passes through G's case analysis */
+    uint64_t levels;           /* passes through G's case analysis, or Euclid steps */
     uint64_t hits_all;         /* large-prime hits the walk visits, before the coprime-m and
                                   stored-x tests (m outside the walked classes are not visited) */
     uint64_t n_small_primes;
     uint64_t n_large_primes;
     uint64_t survivors;        /* set bits in the bitset */
     uint64_t hash;
-    uint64_t bucket_records;   /* hit buckets: stored hits cleared through records (the rest of
-                                  F_large, if any, found their region full and cleared directly) */
+    uint64_t bucket_records;   /* hit buckets: hits cleared through records (of the rest of F_large,
+                                  most are cells that the wheel of d's primes has cleared, which are
+                                  counted only, and any others found their region full) */
 } cs_stats_t;
 
 /* Builds a sieve instance: validates the parameters, computes the row and
