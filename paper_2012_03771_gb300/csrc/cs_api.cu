@@ -16,6 +16,7 @@
 #include "../../include/combsieve.h"
 #include "cs_arith.cuh"
 #include "cs_internal.h"
+#include "cs_prime_bounds.h"
 #include "cs_words.h"
 #include "cs_classes.h"
 
@@ -65,14 +66,6 @@ uint64_t isqrt_u64(uint64_t n) {
     while (r * r > n) r--;
     while ((r + 1) * (r + 1) <= n) r++;
     return r;
-}
-
-// Upper bound on the number of primes in any interval of length y (y >= 2):
-// pi(x + y) - pi(x) <= 2y / log y (Montgomery and Vaughan, "The large sieve",
-// Mathematika 20, 1973), plus slack.
-uint64_t primes_in_interval_bound(uint64_t y) {
-    if (y < 64) return 64;
-    return (uint64_t)(2.0 * (double)y / log((double)y)) + 1024;
 }
 
 // pi(x) < 1.25506 x / log x for x > 1 (Rosser and Schoenfeld, 1962), plus slack.
@@ -148,6 +141,7 @@ struct cs_plan_s {
     std::vector<std::pair<uint64_t, uint64_t>> chunks;    // large-prime ranges (lo, hi]
     std::vector<uint32_t> chunk_seg;                      // m-segments per prime, per chunk
     std::vector<MClasses> chunk_mc;                       // m-classes each chunk walks
+    std::vector<uint64_t> chunk_cap;                      // prime entries per chunk (plans without a cache)
     MClasses mcls = EVERY_M;                              // classes of the chunks with many hits
     MClasses mcls_light = EVERY_M;                        // classes of the other chunks
     uint64_t split_chunks = 0;                            // chunks that walk mcls
@@ -552,7 +546,6 @@ cs_status build_plan(cs_plan_s *pl, uint32_t P, uint64_t d, uint64_t M_start, ui
             pl->split_chunks += mc.Q == pl->mcls.Q && mc.n == pl->mcls.n && pl->mcls.Q > 1;
         }
     };
-    uint64_t widest = 0;
     if (cache) {
         // the cache's chunks that overlap (T, L]; the walk skips primes outside
         ResidueCacheView cv;
@@ -585,16 +578,16 @@ cs_status build_plan(cs_plan_s *pl, uint32_t P, uint64_t d, uint64_t M_start, ui
             // 32-bit kernels
             if (lo < NARROW_LIMIT - 1 && hi >= NARROW_LIMIT) hi = NARROW_LIMIT - 1;
             add_chunk(lo, hi);
-            widest = std::max(widest, hi - lo);
+            pl->chunk_cap.push_back(primes_between_bound(lo, hi));
             lo = hi;
         }
-        pl->large_cap = pl->chunks.empty() ? 0 : primes_in_interval_bound(widest);
+        for (uint64_t n : pl->chunk_cap) pl->large_cap = std::max(pl->large_cap, n);
     }
-    // one segment count and one class choice per chunk (and one cache index
-    // for cached plans): cs_sieve indexes all of them by chunk
+    // one segment count and one class choice per chunk (and one cache index for
+    // cached plans, one entry count for others): cs_sieve indexes all of them by chunk
     const size_t n_chunks = pl->chunks.size();
     if (pl->chunk_seg.size() != n_chunks || pl->chunk_mc.size() != n_chunks ||
-        (pl->cache && pl->cache_idx.size() != n_chunks))
+        (pl->cache ? pl->cache_idx.size() : pl->chunk_cap.size()) != n_chunks)
         return fail(CS_EDEVICE, "internal: large-prime chunk tables disagree");
     pl->small_cap = pl->small_hi > P ? prime_count_bound(pl->small_hi) : 0;
     pl->large_grid = (int)pl->tune.large_grid;   // 0: the launcher picks (one wave of resident CTAs)
@@ -807,13 +800,13 @@ cs_status build_plan(cs_plan_s *pl, uint32_t P, uint64_t d, uint64_t M_start, ui
         if ((s = pl->dalloc(&b, pl->large_cap * el))) return s;
         if ((s = pl->dalloc(&c, pl->large_cap * el))) return s;
         pl->d_lp = a; pl->d_lr = b; pl->d_lv = c;
-        bool any_prep = false;
-        for (size_t k = 0; k < pl->chunks.size(); k++)
-            any_prep = any_prep || (prep_eligible(pl->dp, pl->mode, pl->chunk_seg[k], pl->chunk_mc[k]) &&
-                                    !plan_few(pl, k));
-        if (any_prep && pl->tune.walk_prep != 1) {
-            if ((s = pl->dalloc(&pl->d_desc0, pl->large_cap))) return s;
-            if ((s = pl->dalloc(&pl->d_desc1, pl->large_cap))) return s;
+        uint64_t prep_cap = 0;
+        for (size_t k = 0; k < n_chunks; k++)
+            if (prep_eligible(pl->dp, pl->mode, pl->chunk_seg[k], pl->chunk_mc[k]) && !plan_few(pl, k))
+                prep_cap = std::max(prep_cap, pl->chunk_cap[k]);
+        if (prep_cap && pl->tune.walk_prep != 1) {
+            if ((s = pl->dalloc(&pl->d_desc0, prep_cap))) return s;
+            if ((s = pl->dalloc(&pl->d_desc1, prep_cap))) return s;
         }
     }
     CS_CUDA(cudaEventCreateWithFlags(&pl->done, cudaEventDisableTiming));
@@ -1012,17 +1005,18 @@ cs_status cs_sieve(cs_plan_t pl, void *stream) {
     }
     for (size_t c = 0; c < pl->chunks.size() && !pl->cache; c++) {
         unsigned long long *cnt = pl->d_counts + 1 + c;
+        const uint64_t cap = pl->chunk_cap[c];
         // 32-bit entries and kernels for every chunk below 2^30, also in a plan
         // whose L is above (its buffers hold 64-bit entries, so 32-bit ones fit)
         const bool narrow = pl->narrow || pl->chunks[c].second < NARROW_LIMIT;
         if ((s = prof.begin(KC_GEN_LARGE))) return s;
         CS_CUDA(launch_gen_large(dp, narrow, pl->chunks[c].first, pl->chunks[c].second,
                                  pl->d_base, pl->n_base, pl->d_lp, pl->d_lr, pl->d_lv,
-                                 pl->large_cap, cnt, st));
+                                 cap, cnt, st));
         if ((s = prof.end())) return s;
         if (plan_few(pl, c)) {
             if ((s = prof.begin(KC_LARGE))) return s;
-            CS_CUDA(launch_few(dp, narrow, pl->d_lp, pl->d_lr, pl->d_lv, cnt, pl->large_cap, pl->chunk_mc[c], st));
+            CS_CUDA(launch_few(dp, narrow, pl->d_lp, pl->d_lr, pl->d_lv, cnt, cap, pl->chunk_mc[c], st));
             if ((s = prof.end())) return s;
             if ((s = apply(c))) return s;
             continue;
@@ -1030,13 +1024,13 @@ cs_status cs_sieve(cs_plan_t pl, void *stream) {
         const bool pre = plan_prepares(pl, c);
         if (pre) {
             if ((s = prof.begin(KC_PREP))) return s;
-            CS_CUDA(launch_tg_prep(dp, narrow, pl->d_lp, pl->d_lr, pl->d_lv, cnt, pl->large_cap, 0, ~0ull,
+            CS_CUDA(launch_tg_prep(dp, narrow, pl->d_lp, pl->d_lr, pl->d_lv, cnt, cap, 0, ~0ull,
                                    pl->chunk_mc[c], pl->d_desc0, pl->d_desc1, st));
             if ((s = prof.end())) return s;
         }
         if ((s = prof.begin(KC_LARGE))) return s;
         CS_CUDA(launch_large(dp, narrow, pl->mode, pl->d_lp, pl->d_lr, pl->d_lv, cnt,
-                             pl->large_cap, pl->chunk_seg[c], pl->large_grid, st, 0, ~0ull,
+                             cap, pl->chunk_seg[c], pl->large_grid, st, 0, ~0ull,
                              pl->chunk_mc[c], pre ? pl->d_desc0 : nullptr, pre ? pl->d_desc1 : nullptr));
         if ((s = prof.end())) return s;
         if ((s = apply(c))) return s;

@@ -16,6 +16,7 @@
 
 #include "../../include/combsieve.h"
 #include "cs_internal.h"
+#include "cs_prime_bounds.h"
 
 using namespace cs;
 
@@ -63,25 +64,6 @@ cudaError_t upload_now(void *dst, const void *src, size_t bytes) {
 constexpr uint64_t GRID0 = 1ull << 16;
 constexpr uint64_t GRID_MAX_WIDTH = 1ull << 27;
 constexpr uint64_t NARROW = 1ull << 30;
-
-// pi(x) bounds of P. Dusart (2010): x/ln x (1 + 1/ln x + 2/ln^2 x) <= pi(x) for
-// x >= 88789 and pi(x) <= x/ln x (1 + 1/ln x + 2.51/ln^2 x) for x >= 355991.
-double pi_upper(double x) {
-    if (x < 355991.0) return x < 2 ? 0 : 1.26 * x / log(x) + 16;   // Rosser-Schoenfeld for small x
-    double l = log(x);
-    return x / l * (1 + 1 / l + 2.51 / (l * l));
-}
-double pi_lower(double x) {
-    if (x < 355991.0) return 0;
-    double l = log(x);
-    return x / l * (1 + 1 / l + 2 / (l * l));
-}
-
-uint64_t chunk_cap(uint64_t lo, uint64_t hi) {
-    double c = pi_upper((double)hi) - pi_lower((double)lo);
-    double mv = hi - lo >= 64 ? 2.0 * (double)(hi - lo) / log((double)(hi - lo)) : 64.0;   // Montgomery-Vaughan
-    return (uint64_t)(std::min(c, mv) * 1.01) + 4096;
-}
 
 std::vector<uint32_t> small_primes(uint64_t n) {
     std::vector<uint32_t> out;
@@ -133,7 +115,7 @@ cs_status cache_extend(cs_cache_t c, uint64_t L) {
         ch.lo = lo;
         ch.hi = hi;
         ch.narrow = hi < NARROW;
-        ch.cap = chunk_cap(lo, hi);
+        ch.cap = primes_between_bound(lo, hi);
         const size_t el = ch.narrow ? 4 : 8;
         cs_status s;
         if ((s = c->alloc(&ch.p, ch.cap * el))) return s;
