@@ -570,9 +570,9 @@ cs_status build_plan(cs_plan_s *pl, uint32_t P, uint64_t d, uint64_t M_start, ui
             const MClasses mc = classes_for(lo);
             if (!mc.items && mc.n == 1 && segs_for(lo) == 1) {
                 hi = std::min<uint64_t>(L, lo + chunk);
-                // (few m: up to the primes that take every m)
+                // (few m: up to the primes that try every m)
                 const uint64_t from = few_from(M_inc, S, mc);
-                if (M_inc <= FEW_M && lo < from && from < hi) hi = from;
+                if (lo < from && from < hi) hi = from;
             }
             // a chunk ends below 2^30 when the next one starts above: it keeps the
             // 32-bit kernels

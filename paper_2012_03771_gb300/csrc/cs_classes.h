@@ -80,4 +80,21 @@ inline ClassTiers class_tiers(bool three_gap, uint64_t d, uint64_t M_start, uint
     return ct;
 }
 
+// The light chunks' form for few m: from which prime on trying every m of the class
+// (k_few_m) costs less than a prepared walker (22 to 27 ps a prime for preparation and
+// walk, hardly depending on p).  With n m tried, k_few_m takes 6 + 0.085 n ps and 250 ps
+// for every expected hit, n S / p of them (one GB300, n 1 to 256, S 601 to 50,001, p
+// 2^17 to 2^31: 128 m of S = 50,001 52 ps at p = 2^25, 25 at 2^27, 20 at 2^29; 44 m of
+// 16,001 17, 11 and 10; 256 m of 4001 38, 29 and 27).  That is below 22 ps from p = 25000
+// n S / (1600 - 9 n) on.  Where that prime is below 2^24, the primes under it are too few
+// to be worth a chunk and its three launches, and every prime with at most one
+// expected hit tries every m (22 m of 40,001 to 1e7: 157 us a sieve either way; 128 of
+// 601 124 against 123).
+inline uint64_t few_from(uint64_t M_inc, uint64_t S, const MClasses &mc) {
+    const uint64_t n = (M_inc + mc.Q - 1) / mc.Q;
+    if (9 * n >= 1600) return ~0ull;
+    const uint64_t from = 25000 * n * S / (1600 - 9 * n);
+    return from < (1u << 24) ? n * S : from;
+}
+
 }  // namespace cs

@@ -184,13 +184,8 @@ bool prep_eligible(const DevPlan &pl, int mode, uint32_t n_seg, MClasses mc);
 cudaError_t launch_tg_prep(const DevPlan &pl, bool narrow, const void *p, const void *r, const void *v,
                            const unsigned long long *count, uint64_t cap, uint64_t p_lo, uint64_t p_hi,
                            MClasses mc, uint4 *desc0, uint2 *desc1, cudaStream_t stream);
-// The walk of one-walker chunks over few m (up to FEW_M: one addition per m costs
-// less than the preparation of a walker, about 540 instructions, up to some 200 odd
-// m): every m of the class tried, no preparation, hits cleared directly.  Only for
-// primes above few_from, with at most one expected hit each: the exact tries diverge
-// (230 rows of 503#/210 to 1e7, all m tried: 600 us against 53).
-constexpr uint32_t FEW_M = 256;
-inline uint64_t few_from(uint64_t M_inc, uint64_t S, const MClasses &mc) { return M_inc * S / mc.Q; }
+// The walk of one-walker chunks over few m, for the primes cs_classes.h (few_from)
+// names: every m of the class tried, no preparation, hits cleared directly.
 bool few_eligible(const DevPlan &pl, int mode, uint64_t lo, uint32_t n_seg, MClasses mc);
 cudaError_t launch_few(const DevPlan &pl, bool narrow, const void *p, const void *r, const void *v,
                        const unsigned long long *count, uint64_t cap, MClasses mc, cudaStream_t stream);

@@ -24,6 +24,7 @@
 #include <vector>
 
 #include "cs_arith.cuh"
+#include "cs_classes.h"
 #include "cs_internal.h"
 #include "cs_residue.cuh"
 #include "cs_walker.cuh"
@@ -718,14 +719,13 @@ __global__ void __launch_bounds__(PREP_THREADS) k_tg_prep(const LargeArgs a, uin
     }
 }
 
-// The walk of a chunk of one-walker primes over few m (M_inc <= FEW_M): no steps and
-// no first hit, every walked m is tried.  v / p as a 32-bit fraction of a turn advances
+// The walk of a chunk of one-walker primes over few m (few_from): no steps and no
+// first hit, every walked m is tried.  v / p as a 32-bit fraction of a turn advances
 // by a constant per step and wraps by itself, so a step is an addition and a minimum; m
 // whose fraction, with a margin for the roundings, is at most 2SL / p are then tried
-// exactly.  Bound: instruction issue, about 120 per prime at 22 odd m against 600 of the
-// preparation and the walk's descriptors (for primes with less than one expected hit:
-// the exact tries diverge): 11 rows of 1511#/210 to 1e10, preparation
-// and walk 13.0 ms, this kernel 6.0.
+// exactly.  Bound: instruction issue, 6 ps a prime and 0.085 per m, and 250 ps for each
+// hit, whose warp waits for it.  11 rows of 1511#/210 to 1e10 (22 odd m): preparation and
+// walk 13.0 ms, this kernel 4.1.
 constexpr int FEW_THREADS = 256;
 constexpr int FEW_PASS = 8;
 template <class UT>
@@ -740,20 +740,25 @@ __global__ void __launch_bounds__(FEW_THREADS) k_few_m(const LargeArgs a) {
     // the fractions start within 2 and step within 2
     const uint32_t margin = 2 * n_step + 4;
     const uint64_t stride = (uint64_t)gridDim.x * FEW_THREADS;
+    const unsigned lane = threadIdx.x & 31;
     Counters c;
+    if (n == 0) return;
     UT p_next = 0, r_next = 0, v_next = 0;
     auto load = [&](uint64_t i) {
-        if (i < n) {
-            p_next = Pp[i];
-            r_next = Rp[i];
-            v_next = Vp[i];
-        }
+        i = min(i, n - 1);                                         // lanes past the end repeat a prime
+        p_next = Pp[i];
+        r_next = Rp[i];
+        v_next = Vp[i];
     };
-    const uint64_t i_first = blockIdx.x * (uint64_t)FEW_THREADS + threadIdx.x;
-    load(i_first);
-    for (uint64_t i = i_first; i < n; i += stride) {
+    // a warp takes 32 consecutive primes at a time and its lanes stay together: the tries
+    // of a pass are entered and left by all (a warp once split ran all its later passes
+    // and primes in parts: 97#/15, 256 m, S = 40,001 to 1e9 14.5 ms)
+    uint64_t i0 = blockIdx.x * (uint64_t)FEW_THREADS + threadIdx.x - lane;
+    if (i0 < n) load(i0 + lane);
+    for (; i0 < n; i0 += stride) {
+        const uint64_t i = i0 + lane;
         const UT p = p_next, r = r_next, v0 = v_next;
-        load(i + stride);                                          // in flight meanwhile
+        if (i0 + stride < n) load(i + stride);                     // in flight meanwhile
         const UT v = off0 ? add_times(v0, r, 1, p) : v0;           // off0 < Q <= 2
         const UT rq = Q > 1 ? add_times(r, r, 1, p) : r;
         const float rp = walker_rcp(p);
@@ -770,17 +775,22 @@ __global__ void __launch_bounds__(FEW_THREADS) k_few_m(const LargeArgs a) {
                 low = min(low, u);
             }
             u += du;
-            if (low > top) continue;
-            uint32_t t = start;
-            for (uint32_t j = j0; j < min(j0 + FEW_PASS, n_step); j++, t += du) {
-                if (t > top) continue;
-                const uint64_t vm = ((uint64_t)v + (uint64_t)rq * j) % p;      // j < 2^8
-                if (vm > w) continue;
-                c.hits++;
-                const uint32_t moff = off0 + Q * j, z = w - (uint32_t)vm;
-                if (bit_of(__ldg(&pl.col_mask[z >> 5]), z))
-                    take_hit<UT, false, false>(pl, moff, z, __ldg(&pl.row_tab[moff >> 5]), Pp, (uint32_t)i, c.F, nullptr);
+            const bool open = low <= top && i < n;
+            if (!__any_sync(0xffffffffu, open)) continue;
+            if (open) {
+                uint32_t t = start;
+                for (uint32_t j = j0; j < min(j0 + FEW_PASS, n_step); j++, t += du) {
+                    if (t > top) continue;
+                    const uint64_t vm = ((uint64_t)v + (uint64_t)rq * j) % p;      // j < 2^8
+                    if (vm > w) continue;
+                    c.hits++;
+                    const uint32_t moff = off0 + Q * j, z = w - (uint32_t)vm;
+                    if (bit_of(__ldg(&pl.col_mask[z >> 5]), z))
+                        take_hit<UT, false, false>(pl, moff, z, __ldg(&pl.row_tab[moff >> 5]), Pp, (uint32_t)i, c.F,
+                                                   nullptr);
+                }
             }
+            __syncwarp();
         }
     }
     const unsigned long long F = warp_sum(c.F), hits = warp_sum(c.hits);
@@ -900,7 +910,7 @@ bool prep_eligible(const DevPlan &pl, int mode, uint32_t n_seg, MClasses mc) {
 }
 
 bool few_eligible(const DevPlan &pl, int mode, uint64_t lo, uint32_t n_seg, MClasses mc) {
-    return prep_eligible(pl, mode, n_seg, mc) && pl.M_inc <= FEW_M && lo >= few_from(pl.M_inc, pl.S, mc);
+    return prep_eligible(pl, mode, n_seg, mc) && lo >= few_from(pl.M_inc, pl.S, mc);
 }
 
 cudaError_t launch_few(const DevPlan &pl, bool narrow, const void *p, const void *r, const void *v,
