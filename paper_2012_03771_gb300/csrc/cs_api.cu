@@ -15,6 +15,7 @@
 
 #include "../../include/combsieve.h"
 #include "cs_arith.cuh"
+#include "cs_cost.h"
 #include "cs_internal.h"
 #include "cs_prime_bounds.h"
 #include "cs_words.h"
@@ -649,23 +650,7 @@ cs_status build_plan(cs_plan_s *pl, uint32_t P, uint64_t d, uint64_t M_start, ui
     pl->M_c = M_c; pl->W = W; pl->wpr = wpr; pl->S = S; pl->S32 = S32;
     CS_CUDA(prepare_tile(optin));
 
-    // relative cost, for ordering instances in a batch: tile pairs, walk hits,
-    // large primes (each weighted by its measured per-unit time on a GB300)
-    {
-        auto pi = [](double x) { return x < 3 ? 0.0 : x / std::log(x); };
-        const double Td = (double)T, Ld = (double)std::max<uint64_t>(L, 2);
-        const double small = (double)M_c * std::max(0.0, pi((double)pl->small_hi) - pi((double)P));
-        double hits = 0, large = 0;
-        if (L > T && T > 2) {
-            hits = (double)M_inc * (double)S * std::log(std::log(Ld) / std::log(Td));
-            large = pi(Ld) - pi(Td);
-        }
-        // per-unit times measured on search_953: 7.4 ps per (row, small prime)
-        // pair, ~7 ps per walk hit, ~150 ps per large prime (generation, K mod p
-        // and the walk's solves), ~5 us per kernel launch
-        pl->est_cost = (uint64_t)(small * 7.4 + hits * 7.0 + large * (cache ? 60.0 : 150.0) +
-                                  5e6 * (3.0 + 2.0 * (double)pl->chunks.size()));
-    }
+    pl->est_cost = (uint64_t)sieve_cost_ps(M_c, M_inc, S, P, T, L, klimb.size(), pl->chunks.size(), cache != nullptr);
 
     // device memory and tables
     DevPlan &dp = pl->dp;
