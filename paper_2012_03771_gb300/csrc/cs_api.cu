@@ -575,9 +575,7 @@ cs_status build_plan(cs_plan_s *pl, uint32_t P, uint64_t d, uint64_t M_start, ui
                 const uint64_t from = few_from(M_inc, S, mc);
                 if (lo < from && from < hi) hi = from;
             }
-            // a chunk ends below 2^30 when the next one starts above: it keeps the
-            // 32-bit kernels
-            if (lo < NARROW_LIMIT - 1 && hi >= NARROW_LIMIT) hi = NARROW_LIMIT - 1;
+            hi = chunk_end(lo, hi);
             add_chunk(lo, hi);
             pl->chunk_cap.push_back(primes_between_bound(lo, hi));
             lo = hi;

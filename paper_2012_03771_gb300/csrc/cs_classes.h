@@ -15,6 +15,7 @@
 #include <stdint.h>
 
 #include <algorithm>
+#include <initializer_list>
 #include <numeric>
 #include <vector>
 
@@ -78,6 +79,16 @@ inline ClassTiers class_tiers(bool three_gap, uint64_t d, uint64_t M_start, uint
             if (d % Q == 0 && (Q > 6 || t.m_classes == 3)) ct.fine.push_back(class_items(Q, M_start));
     }
     return ct;
+}
+
+// Where a chunk (lo, hi] of large primes ends: below 2^30 or 2^32 when it would cross
+// it, so that all its primes take one form (32-bit fields below 2^30; of the 64-bit
+// ones, residues with one word per prime below 2^32 and two above, whose float
+// quotients are derived for those ranges).
+inline uint64_t chunk_end(uint64_t lo, uint64_t hi) {
+    for (uint64_t limit : {1ull << 30, 1ull << 32})
+        if (lo < limit - 1 && hi >= limit) return limit - 1;
+    return hi;
 }
 
 // The light chunks' form for few m: from which prime on trying every m of the class

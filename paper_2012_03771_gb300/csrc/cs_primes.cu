@@ -530,8 +530,9 @@ cudaError_t launch_res_kernel(const GenArgs &a, cudaStream_t stream) {
     k_large_res<P32, V><<<sm_count() * per_sm, RES_THREADS, 0, stream>>>(a);
     return cudaGetLastError();
 }
+// (a chunk of a plan or a cache lies below 2^32, which is no prime, or above)
 cudaError_t launch_res(const GenArgs &a, uint64_t hi, bool with_v, cudaStream_t stream) {
-    if (hi >> 32) return with_v ? launch_res_kernel<false, true>(a, stream) : launch_res_kernel<false, false>(a, stream);
+    if (hi > 1ull << 32) return with_v ? launch_res_kernel<false, true>(a, stream) : launch_res_kernel<false, false>(a, stream);
     return with_v ? launch_res_kernel<true, true>(a, stream) : launch_res_kernel<true, false>(a, stream);
 }
 }  // namespace

@@ -2,10 +2,11 @@
 //
 // Exact division by 2^32 (K. Hensel; Montgomery's REDC of a long number): with
 // s = 0, for each limb k_i from the lowest, s <- (s + k_i + m p) / 2^32, where m
-// makes the sum divisible.  After n limbs s = K 2^(-32 n) (mod p): a limb costs three multiplies (two for p < 2^32), against the two full 64-bit
-// products per 64-bit word of a Montgomery product over K's factors.  2^(32 n)
-// is put back by one product with 2^(32 n + 64) mod p, which takes a power of two
-// near 2 n + 64 from float quotients and four squarings.
+// makes the sum divisible.  After n limbs s = K 2^(-32 n) (mod p): a limb costs
+// three multiplies (two for p < 2^32), against the two full 64-bit products per
+// 64-bit word of a Montgomery product over K's factors.  2^(32 n) is put back by
+// one product with 2^(32 n + 64) mod p, which takes a power of two near 2 n + 64
+// from float quotients and four squarings.
 #pragma once
 #include <stdint.h>
 
@@ -13,7 +14,8 @@
 
 namespace cs {
 
-// P32: p < 2^32.  ninv = -p^-1 mod 2^32.
+// P32: 2^28 <= p < 2^32, else 2^32 < p < 2^40 (launch_res picks the form by the chunk,
+// which does not cross 2^32).  ninv = -p^-1 mod 2^32.
 struct ResMod {
     uint64_t p;
     uint32_t p0, p1, ninv;
