@@ -673,11 +673,7 @@ cs_status build_plan(cs_plan_s *pl, uint32_t P, uint64_t d, uint64_t M_start, ui
             dp.n_bands = (uint32_t)b.n_bands;
             dp.n_regions = (uint32_t)b.n_regions;
             dp.region_cap = (uint32_t)b.cap;
-            // records are the hits the wheel leaves
-            double kept = (double)W;
-            for (uint32_t q : wq)
-                if (q <= 11) kept *= 1.0 - 1.0 / (double)q;
-            pl->apply_after = apply_groups(pl->chunks, M_c, (uint64_t)std::ceil(kept), b);
+            pl->apply_after = apply_groups(pl->chunks, M_c, record_columns(W, wq), b);
             for (uint8_t f : pl->apply_after) pl->apply_launches += f;
         }
     }

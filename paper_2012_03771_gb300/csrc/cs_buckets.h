@@ -77,6 +77,16 @@ inline double expected_stored_hits(uint64_t lo, uint64_t hi, uint64_t M_c, uint6
     return (double)M_c * (double)W * std::log(std::log(h) / std::log(l));
 }
 
+// Stored columns of a row that become records when a prime hits them: W less those
+// the wheel's primes up to 11 have cleared (the walk counts a hit there without a
+// clear).
+inline uint64_t record_columns(uint64_t W, const std::vector<uint32_t> &wheel) {
+    double kept = (double)W;
+    for (uint32_t q : wheel)
+        if (q <= 11) kept *= 1.0 - 1.0 / (double)q;
+    return (uint64_t)std::ceil(kept);
+}
+
 // apply_after[c] = 1 when the records are cleared after chunk c's walk: chunks
 // are grouped in order so that a group's expected stored hits fill at most
 // 60% of all regions (a chunk that alone expects more forms its own group, and
