@@ -689,13 +689,10 @@ cs_status build_plan(cs_plan_s *pl, uint32_t P, uint64_t d, uint64_t M_start, ui
     dp.n_kch32 = (uint32_t)kch32.size();
     dp.n_klimb = (uint32_t)klimb.size();
     pl->stage(&dp.col_mask, col_mask);
-    pl->stage(&dp.col_prefix, col_prefix);
     pl->stage(&dp.raw_of_col, raw_of_col);
     pl->stage(&dp.moff_of_row, moff_of_row);
-    pl->stage(&dp.row_mask, row_mask);
-    pl->stage(&dp.row_prefix, row_prefix);
     {
-        // the same tables interleaved as {mask, prefix} pairs for the walk's lookups
+        // the row table, and the column table beside its mask, as {mask, prefix} pairs for the walk's lookups
         std::vector<uint2> ct(S32), rt(row_mask.size());
         for (uint64_t w = 0; w < S32; w++) ct[w] = make_uint2(col_mask[w], col_prefix[w]);
         for (size_t w = 0; w < row_mask.size(); w++) rt[w] = make_uint2(row_mask[w], row_prefix[w]);

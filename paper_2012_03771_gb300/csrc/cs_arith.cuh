@@ -170,6 +170,8 @@ CS_HD uint32_t mont32_rpow(uint32_t e, uint32_t r1, uint32_t r2, uint32_t p, uin
 }
 
 // ---------------------------------------------------------------- R = 2^64
+// (No kernel runs these any more: 64-bit residues come from K's limbs, cs_residue.cuh.
+// The host test of the arithmetic still checks them.)
 CS_HD uint64_t mont64_neg_inv(uint64_t p) {
     uint64_t x = p;
     x *= 2u - p * x;
@@ -237,17 +239,6 @@ CS_HD uint64_t mont64_rpow2(uint32_t e, uint64_t r2, uint64_t p, uint64_t pinv) 
         if (k & 1) acc = mont64_mul(acc, base, p, pinv);
         k >>= 1;
         if (k) base = mont64_mul(base, base, p, pinv);
-    }
-    return acc;
-}
-
-CS_HD uint64_t mont64_rpow(uint32_t e, uint64_t r1, uint64_t r2, uint64_t p, uint64_t pinv) {
-    uint64_t acc = r1, base = r2;
-    uint32_t k = e - 1;
-    while (k) {
-        if (k & 1) acc = mont64_mul(acc, base, p, pinv);
-        base = mont64_mul(base, base, p, pinv);
-        k >>= 1;
     }
     return acc;
 }

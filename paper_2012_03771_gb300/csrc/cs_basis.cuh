@@ -55,13 +55,6 @@ CS_HD float near_fma(float a, float b, float c) {
     return fmaf(a, b, c);
 #endif
 }
-CS_HD float near_sub(float a, float b) {
-#if defined(__CUDA_ARCH__)
-    return __fsub_rn(a, b);
-#else
-    return a - b;
-#endif
-}
 CS_HD int32_t near_int(float sum) { return (int32_t)((uint32_t)float_bits(sum) - 0x4B400000u); }
 
 // float of a signed 64-bit number through its halves: within 2^8 + 2^-22 |x|
