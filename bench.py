@@ -387,7 +387,7 @@ def csrc_sha() -> str:
 
 # ncu counters of the large-prime walk, summed over the walk's launches of one
 # sieve (the first, the bench's warm-up sieve) of each workload, taken with
-#   ncu --metrics smsp__thread_inst_executed.sum,gpu__time_duration.sum --clock-control none
+#   ncu --metrics gpu__time_duration.sum,smsp__thread_inst_executed.sum --clock-control none
 #       -k regex:"k_large_tg|k_tg_prep" -c 1424 --csv python bench.py --steps 1 --warmup 1 --no-cpu
 #   ncu --metrics gpu__time_duration.sum,smsp__thread_inst_executed.sum,dram__bytes_read.sum,
 #       dram__bytes_write.sum --clock-control none -k regex:"k_large_tg|k_tg_prep" -c 24 --csv
@@ -401,12 +401,12 @@ WALK_COUNTERS = {
     # visits (large_1019 buckets its clears, search_953 clears directly); prep_*: the
     # walker-preparation kernel of the same run; large_1019's DRAM bytes were not
     # captured at full size (several passes on a 13 GB working set)
-    "large_1019": {"csrc_sha": "58bfec8b3616bf72", "threshold": 100002, "tile_rows": 8, "launches": 756,
-                   "thread_inst": 9043307908990.0, "dram_bytes": None,
-                   "prep_launches": 668, "prep_thread_inst": 1932755864669.0},
-    "search_953": {"csrc_sha": "58bfec8b3616bf72", "threshold": 120003, "tile_rows": 16, "launches": 17,
-                   "thread_inst": 66209562636.0, "dram_bytes": 1742188544.0,
-                   "prep_launches": 7, "prep_thread_inst": 15563575454.0},
+    "large_1019": {"csrc_sha": "f5c29c0c516be9fa", "threshold": 100002, "tile_rows": 8, "launches": 756,
+                   "thread_inst": 9061932591032.0, "dram_bytes": None,
+                   "prep_launches": 668, "prep_thread_inst": 1940041187510.0},
+    "search_953": {"csrc_sha": "f5c29c0c516be9fa", "threshold": 120003, "tile_rows": 16, "launches": 17,
+                   "thread_inst": 66265169417.0, "dram_bytes": 1741826816.0,
+                   "prep_launches": 7, "prep_thread_inst": 15651275709.0},
 }
 
 
@@ -445,14 +445,32 @@ def clear_rate(torch, cs, stream, words):
         return None
 
 
+def wheel_share(params) -> float:
+    """Share of the cells (row, stored x) that the walk's wheel test leaves (d's primes
+    up to 11): a prime q of d that divides x never divides m K + x, one that does not
+    does for one of the q - 1 classes of m."""
+    import numpy as np
+    x = np.arange(-params.SL, params.SL + 1)
+    stored, share = np.ones(len(x), dtype=bool), np.ones(len(x))
+    for q in range(2, params.P + 1):
+        if any(q % f == 0 for f in range(2, int(q ** 0.5) + 1)):
+            continue
+        if params.d % q:
+            stored[x % q == 0] = False
+        elif q <= 11:
+            share[x % q != 0] *= (q - 2) / (q - 1)
+    return float(share[stored].mean()) if stored.any() else 1.0
+
+
 def roofline(dom, kern_ms, kern_n, stats, info, params, peaks, peak_src, issue, config, clears_peak=None,
              band_peak=None):
     """Roofline of the dominant kernel class over its average CUDA-event launch
     duration (timed on the launching stream).  The large-prime walk has two
     bounds: the integer issue rate (thread instructions per sieve, from stored
-    ncu counters, against cs_issue_rate) and its memory side.  With direct
-    clears that is the scattered bit clears (its stored hits, F_large, counted
-    live, against cs_atomic_rate over a region of the bitset's size); with hit
+    ncu counters, against cs_issue_rate; idle lanes of a warp count in the steps
+    it takes together) and its memory side.  With direct clears that is the
+    scattered bit clears (of its stored hits, counted live, those the wheel
+    leaves, against cs_atomic_rate over a region of the bitset's size); with hit
     buckets it is the 4-byte records it writes (against the measured HBM copy
     rate), and the apply kernel that clears them gets its own entry (records
     counted live, against cs_atomic_rate over a region of two bands).  The
@@ -510,7 +528,8 @@ def roofline(dom, kern_ms, kern_n, stats, info, params, peaks, peak_src, issue, 
                             "peak_source": "measured in this run: cs_atomic_rate over a region of two bands' "
                                            "words (best of three launches)"}
     elif clears_peak:
-        clears_launch = stats["F_large"] / n_chunks           # stored hits: one bit clear each
+        # one bit clear for each stored hit (counted live) that the wheel leaves
+        clears_launch = stats["F_large"] * (wheel_share(params) if params is not None else 1.0) / n_chunks
         achieved = clears_launch / per_launch_s / 1e9
         clears_b = {"achieved": achieved, "peak": clears_peak / 1e9, "unit": "Gclears/s",
                     "frac": achieved / (clears_peak / 1e9), "min_ms_per_launch": clears_launch / clears_peak * 1e3,
@@ -525,8 +544,11 @@ def roofline(dom, kern_ms, kern_n, stats, info, params, peaks, peak_src, issue, 
                        "frac": ach / peak, "ms_per_sieve": prep_s * 1e3, "launches_per_sieve": int(info.prep_chunks)}
     out["launches_timed"] = n_launch
     walk_s = kern_ms[dom] / 1e3 / max(n_launch / n_chunks, 1)   # walk seconds per sieve
+    # ps_per_visited_hit is the figure to compare between versions: the lanes of a warp
+    # step together, so thread instructions count idle lanes in the common steps too
     out["per_unit_rates"] = {"visited_hits_per_s": stats["hits_all"] / walk_s, "levels_per_s": stats["levels"] / walk_s,
-                             "clears_per_s": stats["F_large"] / walk_s}
+                             "stored_hits_per_s": stats["F_large"] / walk_s,
+                             "ps_per_visited_hit": walk_s * 1e12 / max(stats["hits_all"], 1)}
     binding = None
     mem_b = clears_b or records_b
     if issue_b and mem_b:
