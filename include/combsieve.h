@@ -118,7 +118,9 @@ typedef struct {
                                 segment per prime, in a plan without a residue cache): 2 = each
                                 prime's first hit and steps computed by a preparation kernel
                                 into a 24-byte walker descriptor that the walk reads; 1 = the
-                                walk prepares its items itself; 0 = automatic (2) */
+                                walk prepares its items itself; 0 = automatic (2; over few m,
+                                up to about 170 of the walked class, the chunks of rarely hit
+                                primes try every m instead) */
 } cs_tuning;
 
 typedef struct {
@@ -160,8 +162,11 @@ typedef struct {
     uint64_t F;                /* enumerated factors (F_small + F_large) */
     uint64_t F_small;
     uint64_t F_large;
-    uint64_t solves;           /* G solves of Eq. modeq in the large-prime walk */
-    uint64_t levels;           /* passes through G's case analysis, or Euclid steps */
+    uint64_t solves;           /* G solves of Eq. modeq in the large-prime walk (the windows
+                                  whose answer it needs, by whatever way); chunks over few m
+                                  whose every m is tried solve none */
+    uint64_t levels;           /* passes through G's case analysis, or Euclid steps (none in
+                                  those chunks) */
     uint64_t hits_all;         /* large-prime hits the walk visits, before the coprime-m and
                                   stored-x tests (m outside the walked classes are not visited) */
     uint64_t n_small_primes;
@@ -248,11 +253,13 @@ const char *cs_last_error(void);
  * for that threshold and tile height.  The choice is kept
  * per (P, d, SL, ceil(log2 L)) in memory and, if cache_path is not NULL,
  * appended to that text file and read back by later calls (one line per key).
+ * The candidates (tiles of 8 to 32 rows, T of 2 to 16 S) are for searches of
+ * about 5,000 rows and more; for fewer a zeroed tuning is the faster one.
  * *out receives a complete tuning (large_mode = 2).  Validation errors as for
  * cs_plan.  Tuning fields left at 0 in any plan may also be set from the
  * environment: CS_THRESHOLD, CS_TILE_ROWS, CS_LARGE_MODE, CS_LARGE_GRID, CS_M_CLASSES,
  * CS_ITEM_HITS, CS_CLASS_MIN_HITS, CS_CLASS_ITEM_HITS, CS_CHUNK_NUMBERS, CS_HIT_BUCKETS,
- * CS_BAND_ROWS_LOG, CS_BUCKET_RECORDS. */
+ * CS_BAND_ROWS_LOG, CS_BUCKET_RECORDS, CS_WALK_PREP. */
 cs_status cs_autotune(uint32_t P, uint64_t d, uint64_t M_start, uint64_t M_inc, uint32_t SL, uint64_t L,
                       const char *cache_path, cs_tuning *out);
 
@@ -319,7 +326,8 @@ cs_status cs_primes(uint64_t lo, uint64_t hi, uint64_t *out, uint64_t cap, uint6
                     void *stream);
 
 /* r[i] = K mod p[i] for K = P#/d (Section 3.1), for odd p[i] > P, p[i] < 2^40.
- * Montgomery arithmetic with R = 2^32 when p < 2^31, else R = 2^64.
+ * Montgomery products by K's factor words (R = 2^32) when p < 2^31, else exact
+ * division by 2^32 over K's limbs.
  * Synchronises `stream`. */
 cs_status cs_k_mod_p(uint32_t P, uint64_t d, const uint64_t *p, uint64_t n, uint64_t *r,
                      void *stream);

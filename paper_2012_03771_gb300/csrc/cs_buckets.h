@@ -77,9 +77,11 @@ inline double expected_stored_hits(uint64_t lo, uint64_t hi, uint64_t M_c, uint6
     return (double)M_c * (double)W * std::log(std::log(h) / std::log(l));
 }
 
-// Stored columns of a row that become records when a prime hits them: W less those
-// the wheel's primes up to 11 have cleared (the walk counts a hit there without a
-// clear).
+// Stored columns of a row that become records when a prime hits them: W less
+// those the wheel's primes up to 11 have cleared (the walk counts a hit there
+// without a clear).  From above: it takes the columns as independent of those
+// primes, of which they hold the multiples (large_1019: 3814 of 16,682; 0.177 of
+// them, 2959, were counted), so groups end a little early.
 inline uint64_t record_columns(uint64_t W, const std::vector<uint32_t> &wheel) {
     double kept = (double)W;
     for (uint32_t q : wheel)

@@ -236,10 +236,10 @@ __global__ void __launch_bounds__(LARGE_THREADS) k_large(const LargeArgs a) {
 // first hit.  The walk visits a third of the hits (Q = 6) or half of them
 // (Q = 2).  Class items (NC = 1, mc.items classes, Q = 30 or 210): each work
 // item is one class of one (prime, m-segment), so the finer classes (4/15 or
-// 8/35 of the hits) cost one Euclid run per class walker.  The two steps come from one run of Euclid's algorithm on (p, r')
-// (tg_steps, the same answers as G for the two step windows); in the 32-bit
-// walk the first hits follow from the two step vectors, a basis of the lattice
-// of (j, r' j mod p) (first_hit32; first_hit64 in the 64-bit walk).
+// 8/35 of the hits) cost one Euclid run per class walker.  The two steps come from
+// one run of Euclid's algorithm on (p, r') (walker_steps, the same answers as G for
+// the two step windows), the first hits from the two step vectors, a basis of the
+// lattice of (j, r' j mod p) (walker_first_hit).
 // A prepared walker: after its first hit v and the steps of v are at most
 // 2SL < 2^22, so 32 bits hold them for both prime widths; the prime itself is
 // referenced by its index in the chunk's arrays.

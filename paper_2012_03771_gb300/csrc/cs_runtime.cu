@@ -12,7 +12,7 @@
 //   prime chunks run instead as jobs of a few persistent launches (one per walk
 //   kernel, the most costly plans' jobs first) between the plans' tile sieves
 //   and their counts.  That is not the default: on the 64-instance mix it
-//   measured 1.19 s per run against 0.99 s with a launch per chunk, which keeps
+//   measured 627 ms per run against 536 ms with a launch per chunk, which keeps
 //   one chunk's primes and one plan's bitset in L2 at a time and reads the plan
 //   from the kernel parameters.
 // * Server: requests arrive over time; a request is admitted when a slot (a
@@ -118,9 +118,9 @@ cs_status cs_batch_create(const cs_plan_t *plans, int n, int n_streams, cs_batch
     if (!out || !plans || n <= 0) return set_error(CS_EINVAL, "need plans, n >= 1 and out");
     *out = nullptr;
     // default width: instances that each fill the GPU gain little from running
-    // side by side and lose L2 locality (64 uneven searches: 1 stream 1.31x,
-    // 2 streams 1.27x, 16 streams 1.0x over plain launches); the residue-cache
-    // fills, when present, run on streams of their own in any case
+    // side by side and lose L2 locality (64 uneven searches with an earlier walk: 1
+    // stream 1.31x, 2 streams 1.27x, 16 streams 1.0x over plain launches; one stream
+    // 1.23x now); the residue-cache fills, when present, run on streams of their own
     bool any_cache = false;
     for (int i = 0; i < n; i++) any_cache = any_cache || (plans[i] && plan_cache(plans[i]));
     if (n_streams <= 0) n_streams = std::min(n, any_cache ? 1 : 2);

@@ -5,14 +5,18 @@
 // Section 3.2 leaves the threshold open ("naively p > 10 S"; the runtime
 // model's C_mult is about 50).  Here it trades two kernels: the tile sieve costs
 // about M_c per small prime, the walk about M_inc S / p hits plus a few solves
-// per large prime.  Both grow with M_inc at the same rate, so the best T hardly
-// depends on M_inc; it depends on S, on the primes near T and on the GPU.  The
-// tuner therefore times candidate settings on a proxy with the same P, d and SL,
-// M_inc clipped to 1e5 and L to 1e9 (a few tens of milliseconds per run): first
-// T and the tile height together, then the item size for the winner.  The
-// choice is kept per (P, d, SL, ceil(log2 L)) in memory and, if a path is
-// given, in a text file that later processes read back (lines of six fields,
-// without an item size, mean the automatic one).
+// per large prime.  Both grow with M_inc at the same rate, so for searches that
+// fill the GPU the best T hardly depends on M_inc; it depends on S, on the primes
+// near T and on the GPU.  The tuner therefore times candidate settings on a proxy
+// with the same P, d and SL, M_inc clipped to 1e5 and L to 1e9 (a few tens of
+// milliseconds per run): first T and the tile height together, then the item size
+// for the winner.  The choice is kept per (P, d, SL, ceil(log2 L)) in memory and,
+// if a path is given, in a text file that later processes read back (lines of six
+// fields, without an item size, mean the automatic one).  Its tile heights (8, 16,
+// 32) and thresholds (2 to 16 S) are those of such searches: below about 5,000 rows
+// the automatic settings, which also take lower tiles, cut the columns and raise T,
+// are the faster ones (228 rows of 503#/210 to 1e7: 180 us against 229 tuned; 953#/210
+// to 1e9: 228 rows 3.19 ms against 3.35, 4571 rows 4.30 against 4.27).
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdio.h>
@@ -36,7 +40,7 @@ using Key = std::tuple<uint32_t, uint64_t, uint32_t, uint32_t>;   // P, d, SL, c
 struct Choice {
     uint64_t T_over_S_x100;   // threshold as a multiple of S, times 100
     uint32_t tile_rows;
-    uint32_t item_hits;       // walked hits per work item (0: the automatic 128)
+    uint32_t item_hits;       // walked hits per work item (0: the automatic 16 to 128)
 };
 
 std::mutex g_mu;
@@ -135,7 +139,7 @@ extern "C" cs_status cs_autotune(uint32_t P, uint64_t d, uint64_t M_start, uint6
             }
         if (best >= 0) {
             // work-item size for the chosen threshold and tile height (the
-            // automatic 128 is the timing above)
+            // automatic one is the timing above)
             for (uint32_t ih : {32u, 64u, 256u, 512u}) {
                 cs_tuning t{};
                 t.large_mode = 2;

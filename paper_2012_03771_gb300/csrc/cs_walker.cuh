@@ -4,13 +4,13 @@
 // kernel right after K mod p instead, it made that kernel 80 registers wide and
 // the two together 22% slower than apart.)
 //
-// With r' = Q r mod p, the two steps of the walk come from one run of
-// Euclid's algorithm on (p, r') (walker_steps), and the class's first hit from
-// the step basis in O(1) (walker_first_hit): the same work, in the same order
-// and arithmetic, as the walk kernel does for an item it prepares itself, so the
-// results and the solver statistics are identical.  The descriptor: d0 = {first m - M_start (NO_WALKER when no hit
-// falls in the range), v at that m, d_a, u_b}, d1 = {steps of m a Q, b Q,
-// clamped to M_inc}.
+// With r' = Q r mod p, the two steps of the walk come from one run of Euclid's
+// algorithm on (p, r') (walker_steps), and the class's first hit from the step
+// basis in O(1) (walker_first_hit): the same work, in the same order and
+// arithmetic, as the walk kernel does for an item it prepares itself, so the
+// results and the solver statistics are identical.  The descriptor: d0 = {first
+// m - M_start (NO_WALKER when no hit falls in the range), v at that m, d_a, u_b},
+// d1 = {steps of m a Q, b Q, clamped to M_inc}.
 #pragma once
 #include <stdint.h>
 
